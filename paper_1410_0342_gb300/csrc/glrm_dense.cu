@@ -152,61 +152,178 @@ __device__ __forceinline__ unsigned long long fadd2(unsigned long long a, unsign
     return d;
 }
 
+__device__ __forceinline__ unsigned long long fmul2(unsigned long long a, unsigned long long b)
+{
+    unsigned long long d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
+__device__ __forceinline__ unsigned long long dup2(float v) { return pk2(v, v); }
+
+// floor / ceil of two values in [0, 2^22]: the sum with 2^23 rounded down / up
+// is exact to an integer.
+__device__ __forceinline__ unsigned long long floor2(unsigned long long a)
+{
+    unsigned long long d;
+    asm("add.rm.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(dup2(8388608.f)));
+    return fadd2(d, dup2(-8388608.f));
+}
+
+__device__ __forceinline__ unsigned long long ceil2(unsigned long long a)
+{
+    unsigned long long d;
+    asm("add.rp.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(dup2(8388608.f)));
+    return fadd2(d, dup2(-8388608.f));
+}
+
+// Whether a kind's derivative is a whole number of magnitude at most 256 for
+// every entry (hinge 0, +-1; l1 0, +-1; ordinal hinge up to levels - 1): such
+// a derivative is a BF16 value, its mid and lo parts are 0.
+__device__ __forceinline__ bool whole_deriv(int kind, float lev)
+{
+    return kind == kLossHinge || kind == kLossL1 || (kind == kLossOrdinal && lev <= 257.f);
+}
+
 // Losses and derivatives of 16 entries that all lie inside the table and
 // share one loss kind with parameters prm (Huber threshold) and lev (ordinal
-// level count).  Quadratic entries run two at a time in packed FP32.  MISS:
-// a NaN value marks a missing entry, which contributes nothing.
+// level count).  MISS: a NaN value marks a missing entry, which contributes
+// nothing whatever its product.  The passes are bound by the instructions of
+// this block (44 per cell in the gradient and 29 in the loss passes with the
+// scalar branches of loss_deriv_k, the issue slots 40% and the FMA pipe 13%
+// busy), so every kind is written without branches, two entries at a time in
+// packed FP32 where the operation exists in that form:
+//   Huber    c = clamp(x, -d, d) is the derivative, c (x - c / 2) the loss
+//   hinge    a NaN value fails z > 0 and loses against 0 in max(z, 0): the
+//            missing cells need no test
+//   logistic e = exp(-|z|) from 2^t with the rounding of t = -|z| log2 e
+//            carried into a correction, log1p(e) = e P(e) with P the degree-9
+//            minimax polynomial of log1p(e) / e on [0, 1] (Remez exchange,
+//            relative error 4.7e-9), 1 / (1 + e) refined by a Newton step
+//   ordinal  with uc = clamp(u, 1, d): p = (ceil(uc) - a)_+ levels above a and
+//            n = (floor(uc) - a)_- below it are active, never both, so the
+//            derivative is q = p + n and the loss q (u - a - q / 2) + |q| / 2
 template <int KIND, bool MISS>
 __device__ __forceinline__ void dn_block(const float (&u)[16], const float (&a)[16], float prm, float lev,
                                          float (&rr)[16], float &lsum)
 {
-    if constexpr (MISS && KIND == kLossQuad) {
-        // a missing cell's NaN propagates into r and is replaced by 0
-        const unsigned long long m1 = pk2(-1.f, -1.f);
-        unsigned long long acc = pk2(0.f, 0.f);
+    const unsigned long long m1 = dup2(-1.f), mh = dup2(-0.5f);
+    unsigned long long acc = 0ull;
+    // u - a of entries w, w + 1; 0 where the value is missing
+    auto resid = [&](int w) {
+        const unsigned long long x = ffma2(pk2(a[w], a[w + 1]), m1, pk2(u[w], u[w + 1]));
+        if constexpr (!MISS) {
+            return x;
+        } else {
+            float x0, x1;
+            upk2(x, x0, x1);
+            return pk2(a[w] == a[w] ? x0 : 0.f, a[w + 1] == a[w + 1] ? x1 : 0.f);
+        }
+    };
+    if constexpr (KIND == kLossQuad) {
 #pragma unroll
         for (int w = 0; w < 16; w += 2) {
-            float r0, r1;
-            upk2(ffma2(pk2(a[w], a[w + 1]), m1, pk2(u[w], u[w + 1])), r0, r1);  // u - a
-            r0 = a[w] == a[w] ? r0 : 0.f;
-            r1 = a[w + 1] == a[w + 1] ? r1 : 0.f;
-            const unsigned long long r = pk2(r0, r1);
+            const unsigned long long r = resid(w);
             acc = ffma2(r, r, acc);
             upk2(fadd2(r, r), rr[w], rr[w + 1]);
         }
-        float l0, l1;
-        upk2(acc, l0, l1);
-        lsum += l0 + l1;
-    } else if constexpr (MISS) {
-        // the losses tolerate a NaN value (no traps, no loops); its results are replaced by 0
+    } else if constexpr (KIND == kLossHuber) {
+#pragma unroll
+        for (int w = 0; w < 16; w += 2) {
+            const unsigned long long x = resid(w);
+            float x0, x1;
+            upk2(x, x0, x1);
+            rr[w] = fmaxf(fminf(x0, prm), -prm);
+            rr[w + 1] = fmaxf(fminf(x1, prm), -prm);
+            const unsigned long long c = pk2(rr[w], rr[w + 1]);
+            acc = ffma2(c, ffma2(c, mh, x), acc);
+        }
+    } else if constexpr (KIND == kLossHinge) {
+        const unsigned long long one = dup2(1.f);
+#pragma unroll
+        for (int w = 0; w < 16; w += 2) {
+            const unsigned long long na = fmul2(pk2(a[w], a[w + 1]), m1);
+            float n0, n1, z0, z1;
+            upk2(na, n0, n1);
+            upk2(ffma2(na, pk2(u[w], u[w + 1]), one), z0, z1);
+            rr[w] = z0 > 0.f ? n0 : 0.f;
+            rr[w + 1] = z1 > 0.f ? n1 : 0.f;
+            acc = fadd2(acc, pk2(fmaxf(z0, 0.f), fmaxf(z1, 0.f)));
+        }
+    } else if constexpr (KIND == kLossLogistic) {
+        constexpr float kP[10] = {1.0f, -0.4999990165233612f, 0.3332996368408203f, -0.24954132735729218f,
+                                  0.19675935804843903f, -0.1530558466911316f, 0.10603641718626022f,
+                                  -0.05695941299200058f, 0.019851399585604668f, -0.0032440118957310915f};
+        const unsigned long long one = dup2(1.f);
+#pragma unroll
+        for (int w = 0; w < 16; w += 2) {
+            const unsigned long long na = fmul2(pk2(a[w], a[w + 1]), m1);
+            const unsigned long long z = fmul2(na, pk2(u[w], u[w + 1]));
+            float z0, z1, y0, y1;
+            upk2(z, z0, z1);
+            // -|z|, not below the logarithm of the smallest normal value; a NaN stays one
+            asm("max.NaN.f32 %0, %1, %2;" : "=f"(y0) : "f"(-fabsf(z0)), "f"(-87.336544f));
+            asm("max.NaN.f32 %0, %1, %2;" : "=f"(y1) : "f"(-fabsf(z1)), "f"(-87.336544f));
+            const unsigned long long y = pk2(y0, y1);
+            const unsigned long long t = fmul2(y, dup2(1.44269502f));  // log2 e = 1.44269502 + 1.92596303e-8
+            unsigned long long lo = ffma2(y, dup2(1.44269502f), fmul2(t, m1));
+            lo = ffma2(y, dup2(1.92596303e-8f), lo);
+            float t0, t1, e0, e1;
+            upk2(t, t0, t1);
+            asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(t0));
+            asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(t1));
+            unsigned long long e = pk2(e0, e1);
+            e = ffma2(fmul2(e, dup2(0.693147182f)), lo, e);
+            const unsigned long long v = fadd2(e, one);
+            float v0, v1, r0, r1;
+            upk2(v, v0, v1);
+            asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(v0));
+            asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r1) : "f"(v1));
+            unsigned long long r = pk2(r0, r1);
+            r = ffma2(r, ffma2(fmul2(v, m1), r, one), r);
+            unsigned long long P = dup2(kP[9]);
+#pragma unroll
+            for (int c = 8; c >= 0; --c) P = ffma2(P, e, dup2(kP[c]));
+            float L0, L1, d0, d1, s0, s1;
+            upk2(ffma2(e, P, pk2(fmaxf(z0, 0.f), fmaxf(z1, 0.f))), L0, L1);
+            upk2(r, r0, r1);
+            upk2(fmul2(e, r), s0, s1);
+            upk2(fmul2(na, pk2(z0 >= 0.f ? r0 : s0, z1 >= 0.f ? r1 : s1)), d0, d1);
+            const bool ok0 = !MISS || a[w] == a[w], ok1 = !MISS || a[w + 1] == a[w + 1];
+            rr[w] = ok0 ? d0 : 0.f;
+            rr[w + 1] = ok1 ? d1 : 0.f;
+            acc = fadd2(acc, pk2(ok0 ? L0 : 0.f, ok1 ? L1 : 0.f));
+        }
+    } else if constexpr (KIND == kLossOrdinal) {
+#pragma unroll
+        for (int w = 0; w < 16; w += 2) {
+            const unsigned long long uc =
+                pk2(fminf(fmaxf(u[w], 1.f), lev), fminf(fmaxf(u[w + 1], 1.f), lev));
+            const unsigned long long av = pk2(a[w], a[w + 1]);
+            float p0, p1, n0, n1;
+            upk2(ffma2(av, m1, ceil2(uc)), p0, p1);
+            upk2(ffma2(av, m1, floor2(uc)), n0, n1);
+            const unsigned long long p = pk2(fmaxf(p0, 0.f), fmaxf(p1, 0.f));  // 0 for a NaN value
+            const unsigned long long n = pk2(fminf(n0, 0.f), fminf(n1, 0.f));
+            const unsigned long long q = fadd2(p, n);
+            acc = ffma2(q, ffma2(q, mh, resid(w)), acc);
+            acc = ffma2(p, dup2(0.5f), acc);
+            acc = ffma2(n, mh, acc);
+            upk2(q, rr[w], rr[w + 1]);
+        }
+    } else {
 #pragma unroll
         for (int w = 0; w < 16; ++w) {
-            const bool v = a[w] == a[w];
+            const bool v = !MISS || a[w] == a[w];
             float L;
             const float d = loss_deriv_k<KIND, float>(u[w], a[w], prm, lev, L);
             lsum += v ? L : 0.f;
             rr[w] = v ? d : 0.f;
         }
-    } else if constexpr (KIND == kLossQuad) {
-        const unsigned long long m1 = pk2(-1.f, -1.f);
-        unsigned long long acc = pk2(0.f, 0.f);
-#pragma unroll
-        for (int w = 0; w < 16; w += 2) {
-            const unsigned long long r = ffma2(pk2(a[w], a[w + 1]), m1, pk2(u[w], u[w + 1]));  // u - a
-            acc = ffma2(r, r, acc);
-            upk2(fadd2(r, r), rr[w], rr[w + 1]);
-        }
-        float l0, l1;
-        upk2(acc, l0, l1);
-        lsum += l0 + l1;
-    } else {
-#pragma unroll
-        for (int w = 0; w < 16; ++w) {
-            float L;
-            rr[w] = loss_deriv_k<KIND, float>(u[w], a[w], prm, lev, L);
-            lsum += L;
-        }
     }
+    float l0, l1;
+    upk2(acc, l0, l1);
+    lsum += l0 + l1;
 }
 
 // Any mix of kinds; entries outside the table (bit clear in `valid`) and
@@ -325,11 +442,16 @@ dense_pass_kernel(const DenseArgs p, const __grid_constant__ CUtensorMap amap)
     if (!XSTEP && own_ok) myspec = p.lossf[own];
     // Y-step with column weights: this thread's column's weight
     const float wown = (!XSTEP && WGT && own_ok) ? p.wcol[own] : 1.f;
+    // (a block past the table's last column: lane 0 is inside, the lanes outside
+    // take its kind and parameters)
     int wkind = -1;
+    bool wwhole = false;
     if constexpr (!XSTEP) {
-        const int kd = __float_as_int(myspec.x);
-        const int k0 = __shfl_sync(0xffffffffu, kd, 0);
-        wkind = __all_sync(0xffffffffu, kd == k0) ? k0 : -1;
+        const int k0 = __shfl_sync(0xffffffffu, __float_as_int(myspec.x), 0);
+        const float y0 = __shfl_sync(0xffffffffu, myspec.y, 0), z0 = __shfl_sync(0xffffffffu, myspec.z, 0);
+        if (!own_ok) myspec = make_float4(__int_as_float(k0), y0, z0, 0.f);
+        wkind = __all_sync(0xffffffffu, __float_as_int(myspec.x) == k0) ? k0 : -1;
+        wwhole = __all_sync(0xffffffffu, whole_deriv(__float_as_int(myspec.x), myspec.z));
     }
     tc_fence_before();
     __syncthreads();
@@ -523,27 +645,25 @@ dense_pass_kernel(const DenseArgs p, const __grid_constant__ CUtensorMap amap)
             }
         }
     } else {
-        for (int it = 0; it < nq; ++it) {
-            const int64_t q = qb + it;
+        // ring positions and phases of the A and loss-table stages, kept as
+        // counters (a chunk is about 250 instructions of a warp: a division
+        // by the stage count would be a tenth of them)
+        int sA = 0, sL = 0;
+        unsigned phA = 0, phL = 0;
+        const bool own_all = __all_sync(0xffffffffu, own_ok), own_any = __any_sync(0xffffffffu, own_ok);
+        int64_t left = p.nother - qb * kDnNT - tb;  // entries of the other dimension from this warp's first on
+        for (int it = 0; it < nq; ++it, left -= kDnNT) {
             const int b = it & 1;
-            const int sA = it % nA;
-            ok = ok && mbar_wait_bounded(&barG1[b], (unsigned)(it >> 1) & 1u);
-            if (XSTEP) ok = ok && mbar_wait_bounded(&barL[it % 3], (unsigned)(it / 3) & 1u);  // loss table
-            ok = ok && mbar_wait_bounded(&barA[sA], (unsigned)(it / nA) & 1u);
-            tc_fence_after();
-            ok = __all_sync(0xffffffffu, ok);  // tcgen05.ld / st below are warp-collective
-            if (!ok) break;
+            // the A tile (and the loss table) lands chunks ahead: its values
+            // are read before the wait for U
+            if (XSTEP) ok = ok && mbar_wait_bounded(&barL[sL], phL);
+            ok = ok && mbar_wait_bounded(&barA[sA], phA);
             float lsum = 0.f;
             float rr[16];
+            bool whole = false;  // every derivative is a whole number BF16 holds
             {
                 const unsigned char *as = ast + sA * SM::a;
-                const int64_t t0 = q * kDnNT;
                 float u[16], a[16];
-                tmem_ld16(taddr + lane_base + (uint32_t)(b * kDnNT + tb), u);
-                // U of this chunk is in registers: its buffer may take the next GEMM1
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&barU[b]);
                 if constexpr (XSTEP) {
                     // box tb / 32, row orow: 16-byte units (tb % 32) / 4 .. + 3, swizzled
                     const unsigned char *row = as + (tb >> 5) * (SM::a / 2) + orow * 128;
@@ -562,32 +682,64 @@ dense_pass_kernel(const DenseArgs p, const __grid_constant__ CUtensorMap amap)
 #pragma unroll
                     for (int w = 0; w < 16; ++w) a[w] = af[(tb + w) * 32 + lane];
                 }
-                const int64_t nv = p.nother - t0 - tb;  // valid columns from tb on
-                const uint32_t valid = !own_ok ? 0u : (nv >= 16 ? 0xffffu : (nv <= 0 ? 0u : (1u << nv) - 1u));
-                const LossF *lf = reinterpret_cast<const LossF *>(lsst + (it % 3) * SM::ls) + tb;
+                ok = ok && mbar_wait_bounded(&barG1[b], (unsigned)(it >> 1) & 1u);
+                tc_fence_after();
+                ok = __all_sync(0xffffffffu, ok);  // tcgen05.ld / st below are warp-collective
+                if (!ok) break;
+                tmem_ld16(taddr + lane_base + (uint32_t)(b * kDnNT + tb), u);
+                // U of this chunk is in registers: its buffer may take the next GEMM1
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&barU[b]);
+                const bool full = own_all && left >= 16;
+                const uint32_t valid =
+                    !own_ok ? 0u : (left >= 16 ? 0xffffu : (left <= 0 ? 0u : (1u << left) - 1u));
+                const LossF *lf = reinterpret_cast<const LossF *>(lsst + sL * SM::ls) + tb;
                 // the kind (and parameters) the 16 entries share, -1 if they do not:
                 // X-step, kept in the w of each column's loss; Y-step, the warp's columns
                 int kind = wkind;
                 float prm = myspec.y, lev = myspec.z;
                 if constexpr (XSTEP) {
                     const LossF l0 = lf[0];
-                    kind = nv > 0 ? __float_as_int(l0.w) : -1;
+                    kind = left > 0 ? __float_as_int(l0.w) : -1;
                     prm = l0.y;
                     lev = l0.z;
                 }
-                if constexpr (XSTEP && WGT) {
-                    dn_block_w(u, a, lf, p.wcol + t0 + tb, valid, rr, lsum);
-                } else if (__all_sync(0xffffffffu, valid == 0xffffu)) {
-                    switch (kind) {
-                    case kLossQuad: dn_block<kLossQuad, MISS>(u, a, prm, lev, rr, lsum); break;
-                    case kLossHuber: dn_block<kLossHuber, MISS>(u, a, prm, lev, rr, lsum); break;
-                    case kLossHinge: dn_block<kLossHinge, MISS>(u, a, prm, lev, rr, lsum); break;
-                    case kLossLogistic: dn_block<kLossLogistic, MISS>(u, a, prm, lev, rr, lsum); break;
-                    case kLossOrdinal: dn_block<kLossOrdinal, MISS>(u, a, prm, lev, rr, lsum); break;
-                    default: dn_block_any<XSTEP>(u, a, lf, myspec, valid, rr, lsum); break;
-                    }
-                } else {
+                if (XSTEP && WGT) {
+                    if constexpr (XSTEP && WGT)
+                        dn_block_w(u, a, lf, p.wcol + (qb + it) * kDnNT + tb, valid, rr, lsum);
+                } else if (!own_any || left <= 0) {  // nothing of this warp lies inside the table
+#pragma unroll
+                    for (int w = 0; w < 16; ++w) rr[w] = 0.f;
+                    whole = true;
+                } else if (kind < 0) {
                     dn_block_any<XSTEP>(u, a, lf, myspec, valid, rr, lsum);
+                } else {
+                    whole = !WGT && (XSTEP ? whole_deriv(kind, lev) : wwhole);
+                    if (!full) {  // cells outside the table count as missing
+#pragma unroll
+                        for (int w = 0; w < 16; ++w)
+                            if (!((valid >> w) & 1u)) a[w] = __int_as_float(0x7fffffff);
+                    }
+                    if (MISS || !full) {
+                        switch (kind) {
+                        case kLossQuad: dn_block<kLossQuad, true>(u, a, prm, lev, rr, lsum); break;
+                        case kLossHuber: dn_block<kLossHuber, true>(u, a, prm, lev, rr, lsum); break;
+                        case kLossHinge: dn_block<kLossHinge, true>(u, a, prm, lev, rr, lsum); break;
+                        case kLossLogistic: dn_block<kLossLogistic, true>(u, a, prm, lev, rr, lsum); break;
+                        case kLossOrdinal: dn_block<kLossOrdinal, true>(u, a, prm, lev, rr, lsum); break;
+                        default: dn_block_any<XSTEP>(u, a, lf, myspec, valid, rr, lsum); break;
+                        }
+                    } else {
+                        switch (kind) {
+                        case kLossQuad: dn_block<kLossQuad, false>(u, a, prm, lev, rr, lsum); break;
+                        case kLossHuber: dn_block<kLossHuber, false>(u, a, prm, lev, rr, lsum); break;
+                        case kLossHinge: dn_block<kLossHinge, false>(u, a, prm, lev, rr, lsum); break;
+                        case kLossLogistic: dn_block<kLossLogistic, false>(u, a, prm, lev, rr, lsum); break;
+                        case kLossOrdinal: dn_block<kLossOrdinal, false>(u, a, prm, lev, rr, lsum); break;
+                        default: dn_block_any<XSTEP>(u, a, lf, myspec, valid, rr, lsum); break;
+                        }
+                    }
                 }
                 if constexpr (!XSTEP && WGT) {  // the column's weight on its 16 entries
                     lsum *= wown;
@@ -611,26 +763,29 @@ dense_pass_kernel(const DenseArgs p, const __grid_constant__ CUtensorMap amap)
                 if (!ok) break;
                 uint32_t hi[8], mi[8], lo[8];
                 const unsigned long long m1 = pk2(-1.f, -1.f);
-                if constexpr (B16) {
+                if (B16 || whole) {  // (whole: warp-uniform) the high parts are all of R
 #pragma unroll
-                    for (int w = 0; w < 16; w += 2) hi[w / 2] = bf2_bits(__floats2bfloat162_rn(rr[w], rr[w + 1]));
+                    for (int w = 0; w < 16; w += 2) {
+                        hi[w / 2] = bf2_bits(__floats2bfloat162_rn(rr[w], rr[w + 1]));
+                        mi[w / 2] = lo[w / 2] = 0u;
+                    }
                 } else {
 #pragma unroll
-                for (int w = 0; w < 16; w += 2) {
-                    // r = hi + mid + lo, each remainder exact in FP32
-                    const __nv_bfloat162 h2 = __floats2bfloat162_rn(rr[w], rr[w + 1]);
-                    const float2 hf = __bfloat1622float2(h2);
-                    const unsigned long long r1 = ffma2(pk2(hf.x, hf.y), m1, pk2(rr[w], rr[w + 1]));
-                    float a0, a1;
-                    upk2(r1, a0, a1);
-                    const __nv_bfloat162 m2 = __floats2bfloat162_rn(a0, a1);
-                    const float2 mf = __bfloat1622float2(m2);
-                    float b0, b1;
-                    upk2(ffma2(pk2(mf.x, mf.y), m1, r1), b0, b1);
-                    hi[w / 2] = bf2_bits(h2);
-                    mi[w / 2] = bf2_bits(m2);
-                    lo[w / 2] = bf2_bits(__floats2bfloat162_rn(b0, b1));
-                }
+                    for (int w = 0; w < 16; w += 2) {
+                        // r = hi + mid + lo, each remainder exact in FP32
+                        const __nv_bfloat162 h2 = __floats2bfloat162_rn(rr[w], rr[w + 1]);
+                        const float2 hf = __bfloat1622float2(h2);
+                        const unsigned long long r1 = ffma2(pk2(hf.x, hf.y), m1, pk2(rr[w], rr[w + 1]));
+                        float a0, a1;
+                        upk2(r1, a0, a1);
+                        const __nv_bfloat162 m2 = __floats2bfloat162_rn(a0, a1);
+                        const float2 mf = __bfloat1622float2(m2);
+                        float b0, b1;
+                        upk2(ffma2(pk2(mf.x, mf.y), m1, r1), b0, b1);
+                        hi[w / 2] = bf2_bits(h2);
+                        mi[w / 2] = bf2_bits(m2);
+                        lo[w / 2] = bf2_bits(__floats2bfloat162_rn(b0, b1));
+                    }
                 }
                 const uint32_t rcol = kDnColR + (uint32_t)(b * 96 + tb / 2);
                 tmem_st8(taddr + lane_base + rcol, hi);
@@ -643,6 +798,14 @@ dense_pass_kernel(const DenseArgs p, const __grid_constant__ CUtensorMap amap)
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&barE[it & 3]);
+            if (++sA == nA) {
+                sA = 0;
+                phA ^= 1u;
+            }
+            if (XSTEP && ++sL == 3) {
+                sL = 0;
+                phL ^= 1u;
+            }
         }
         if (GRAD && ok) {
             ok = mbar_wait_bounded(&barG2[(nq - 1) & 1], (unsigned)((nq - 1) >> 1) & 1u);
@@ -923,35 +1086,35 @@ cudaError_t dense_pack(glrm_s *h, const float *W, int64_t rows)
 }
 
 // Relative cost of evaluating one entry of a 16- or 32-wide group of columns
-// (counted instructions of the loss blocks plus the per-entry load and sum
-// work): a group whose columns share one kind takes that kind's block; a
-// group that mixes kinds, or runs past the table, takes the per-entry switch
-// and pays for every kind present (its lanes diverge).
+// (instructions of the loss blocks, the split of R and the per-entry load and
+// sum work): a group whose columns share one kind takes that kind's block; a
+// group that mixes kinds takes the per-entry switch and pays for every kind
+// present (its lanes diverge).
 double group_cost(const std::vector<LossSpec> &loss, int64_t j0, int width)
 {
     auto extra = [](int kind) -> double {
         switch (kind) {
-        case kLossQuad: return 2;
-        case kLossHuber: return 8;
+        case kLossQuad: return 6;
+        case kLossHuber: return 9;
         case kLossHinge: return 4;
-        case kLossLogistic: return 22;
-        case kLossL1: return 5;
-        case kLossQuantile: return 6;
-        default: return 16;
+        case kLossLogistic: return 24;
+        case kLossL1: return 8;
+        case kLossQuantile: return 10;
+        default: return 12;
         }
     };
-    const int64_t n = (int64_t)loss.size();
-    bool uniform = j0 + width <= n;
+    const int64_t n = (int64_t)loss.size(), j1 = std::min<int64_t>(n, j0 + width);
+    bool uniform = true;
     unsigned seen = 0;
-    for (int64_t j = j0; j < j0 + width; ++j) {
-        const int kd = j < n ? loss[j].kind : kLossQuad;  // lanes past the table run the quadratic block
-        if (j < n && kd != loss[j0].kind) uniform = false;
-        seen |= 1u << kd;
+    for (int64_t j = j0; j < j1; ++j) {
+        if (loss[j].kind != loss[j0].kind) uniform = false;
+        seen |= 1u << loss[j].kind;
     }
+    if (j0 >= j1) return 6;
     if (uniform) return 6 + extra(loss[j0].kind);
-    double c = 10;
+    double c = 16;
     for (int kd = 0; kd < kLossKinds; ++kd)
-        if (seen >> kd & 1u) c += extra(kd);
+        if (seen >> kd & 1u) c += 2 * extra(kd);
     return c;
 }
 
