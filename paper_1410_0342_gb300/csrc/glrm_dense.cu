@@ -27,12 +27,12 @@
 //
 // Pipeline of one CTA (one lane each of three producer warps issues the
 // GEMM1 MMAs, the copies and the GEMM2 MMAs; 16 warps run the per-entry
-// work): GEMM1 runs two chunks ahead into a double-buffered accumulator, so
-// the tensor core computes U of chunk q + 1 while the warps evaluate the
-// losses of chunk q; R is double-buffered in tensor memory, so the warps
-// write R of chunk q while GEMM2 of chunk q - 1 still reads the other buffer;
-// W's GEMM1 and GEMM2 parts are triple-buffered, the A tiles two to four
-// times.
+// work): GEMM1 runs up to two chunks ahead into a double-buffered
+// accumulator, so the tensor core computes U of chunk q + 1 while the warps
+// evaluate the losses of chunk q; R is double-buffered in tensor memory, so
+// the warps write R of chunk q while GEMM2 of chunk q - 1 still reads the
+// other buffer; W's GEMM1 and GEMM2 parts are triple-buffered, the A tiles two
+// to four times.
 #include <cuda.h>
 
 #include <string.h>
@@ -52,11 +52,12 @@ constexpr int kDnNT = 64;        // chunk of the other dimension (UMMA N of GEMM
 constexpr int kDnRows = 128;     // own rows per CTA (UMMA M)
 constexpr int kDnWarps = 16;     // evaluating warp w: TMEM lanes 32 (w % 4) .. + 31, chunk columns 16 (w / 4) .. + 15
 constexpr int kDnThreads = (kDnWarps + 3) * 32;  // + the GEMM1 warp, the copy warp, the GEMM2 warp
-// TMEM columns: U at [0, 64) and [64, 128), G at [128, 128 + KP), two buffers
-// of R (hi, mid, lo; 32 columns each) at [192, 288) and [288, 384), the own
-// rows (hi, mid, lo; KP / 2 columns each) from 384
+// TMEM columns: U at [0, 64) and [64, 128), two buffers of R (hi, mid, lo; 32
+// columns each) at [128, 224) and [224, 320), G from 320 (one block of KP
+// columns per part of W that gets its own accumulator, see DnG), the own rows
+// (hi, mid, lo; KP / 2 columns each) behind it
 constexpr int kDnTmem = 512;
-constexpr int kDnColG = 128, kDnColR = 192, kDnColOwn = 384;
+constexpr int kDnColR = 128, kDnColG = 320;
 constexpr int kDnMaxStages = 4;
 
 // Column loss with its parameters in FP32 (kind as int bits, Huber
@@ -81,17 +82,31 @@ struct DenseArgs {
     int *err;
 };
 
+// GEMM2's accumulator blocks.  An MMA costs the tensor pipe the same from
+// N = 16 up to about N = 128 (44 cycles on an idle SM, measured), so the six
+// products R.part x W.part of a 16-row K step are issued as three MMAs with
+// W's parts side by side in N: R.hi x [hi | mid | lo], R.mid x [hi | mid] and
+// R.lo x [hi], each W part with its own KP columns of G, added at the end.
+// For KP = 64 that would take 192 columns, more than tensor memory has left:
+// there the hi and mid parts are separate MMAs into one block.
+template <int KP>
+struct DnG {
+    static constexpr int NB = KP <= 32 ? 3 : 1;  // blocks
+    static constexpr int Own = kDnColG + NB * KP;
+    static_assert(Own + 3 * KP / 2 <= kDnTmem, "tensor memory");
+};
+
 // Dynamic shared memory of one CTA: the A stages first (1024-byte aligned for
 // the swizzled boxes; 1024 bytes of slack align the base), then three stages
-// of W's three GEMM1 parts, three stages of W's three GEMM2 parts and three
-// stages of the loss table (every operand buffer on a 1024-byte boundary).
+// of W's three GEMM1 parts, three stages of W's three GEMM2 parts and one loss
+// table per A stage (every operand buffer on a 1024-byte boundary).
 template <bool XSTEP, bool GRAD, int KP>
 struct DnSmem {
     static constexpr size_t pk = (size_t)kDnNT * KP * 2;
     static constexpr size_t pt = GRAD ? (size_t)KP * kDnNT * 2 : 0;
     static constexpr size_t ls = XSTEP ? (size_t)kDnNT * sizeof(LossF) : 0;
     static constexpr size_t a = (size_t)kDnNT * kDnRows * 4;  // 32 KB A tile
-    static constexpr size_t fixed = 9 * pk + 9 * pt + 3 * ls;
+    static constexpr size_t fixed = 9 * pk + 9 * pt + kDnMaxStages * ls;
     static size_t bytes(int nA) { return 1024 + fixed + (size_t)nA * a; }
 };
 
@@ -326,16 +341,30 @@ __device__ __forceinline__ void dn_block(const float (&u)[16], const float (&a)[
     lsum += l0 + l1;
 }
 
-// Any mix of kinds; entries outside the table (bit clear in `valid`) and
-// missing entries (NaN) give 0.
-// X-step: the entries are 16 columns (losses in lf); Y-step: one column (own).
-template <bool XSTEP>
+template <bool MISS>
+__device__ __forceinline__ void dn_block_kind(int kind, const float (&u)[16], const float (&a)[16], float prm,
+                                              float lev, float (&rr)[16], float &lsum)
+{
+    switch (kind) {
+    case kLossQuad: dn_block<kLossQuad, MISS>(u, a, prm, lev, rr, lsum); break;
+    case kLossHuber: dn_block<kLossHuber, MISS>(u, a, prm, lev, rr, lsum); break;
+    case kLossHinge: dn_block<kLossHinge, MISS>(u, a, prm, lev, rr, lsum); break;
+    case kLossLogistic: dn_block<kLossLogistic, MISS>(u, a, prm, lev, rr, lsum); break;
+    case kLossOrdinal: dn_block<kLossOrdinal, MISS>(u, a, prm, lev, rr, lsum); break;
+    case kLossL1: dn_block<kLossL1, MISS>(u, a, prm, lev, rr, lsum); break;
+    default: dn_block<kLossQuantile, MISS>(u, a, prm, lev, rr, lsum); break;
+    }
+}
+
+// The X-step with any mix of kinds: the entries are 16 columns (losses in lf;
+// the branches are uniform over the warp); entries outside the table (bit
+// clear in `valid`) and missing entries (NaN) give 0.
 __device__ __forceinline__ void dn_block_any(const float (&u)[16], const float (&a)[16], const LossF *lf,
-                                             LossF own, uint32_t valid, float (&rr)[16], float &lsum)
+                                             uint32_t valid, float (&rr)[16], float &lsum)
 {
 #pragma unroll
     for (int w = 0; w < 16; ++w) {
-        const LossF sp = XSTEP ? lf[w] : own;
+        const LossF sp = lf[w];
         float L;
         const float d = loss_deriv_kind<float>(__float_as_int(sp.x), u[w], a[w], sp.y, sp.z, L);
         const bool v = ((valid >> w) & 1u) && a[w] == a[w];
@@ -368,19 +397,34 @@ __device__ __forceinline__ void dn_block_w(const float (&u)[16], const float (&a
 // A tiles: X-step, two boxes of 32 columns x 128 own rows with the 128-byte
 // swizzle (16-byte unit u of row r at u ^ (r % 8): conflict-free row reads);
 // Y-step, one box of 128 own columns x 64 rows, unswizzled.
-// Warps 0 .. 15 evaluate the entries; lane 0 of warp 16 issues the MMAs (and
-// the copies of W's GEMM1 parts), lane 0 of warp 17 the other copies.  The
-// MMA warp learns from barU[c % 2] (one arrival per evaluating warp) that U of
-// chunk c has been read out of tensor memory and issues GEMM1 of chunk c + 2
-// into that buffer at once; both learn from barE[c % 4] that the entries of
-// chunk c are done (A stage read, R written): the copy warp refills the
-// stages, the MMA warp issues GEMM2.  The evaluating warps never wait for each
-// other inside the loop.  A warp can start chunk c only after every warp has
-// read U of chunk c - 2, so after every warp has finished chunk c - 3: four
-// barE barriers keep the arrivals of different chunks apart, and neither
-// producer warp can fall two phases behind a barrier it waits on (the copy
-// warp issues the A tile every chunk c needs after the wait for chunk c - 4
-// at the latest; the MMA warp issues GEMM1 of c after its wait for c - 2).
+// Warps 0 .. 15 evaluate the entries; one lane each of warp 16 issues GEMM1,
+// of warp 17 the copies, of warp 18 GEMM2 (two warps: beside four evaluating
+// warps on its scheduler an issuing warp spends 70 to 170 cycles per MMA, and
+// both GEMMs of a chunk from one warp took longer than its evaluation).
+// A warp's chunk is a chain of latencies (tensor memory load, shared-memory
+// load, barrier polls) and only four warps share a scheduler, so the loads of
+// chunk c + 1 are started in the middle of chunk c, as soon as its losses are
+// formed (the registers of U and A are free then), and land behind the split
+// and the stores of R.
+// barU[c % 4]: every warp holds U of chunk c in registers; the GEMM1 warp
+// issues GEMM1 of c + 2 into that accumulator, the copy warp W's part of c + 3
+// into the stage GEMM1 of c has read.  barE[c % 4]: the entries of chunk c are
+// done (A stage read, R written); the GEMM2 warp issues GEMM2 of c, the copy
+// warp refills the A stage.  barG1[c % 2] completes when GEMM1 of chunk c is
+// done, the copy warp has seen A of c land (with two A stages the tile is
+// requested too late for that: the evaluating warps poll barA themselves) and
+// the GEMM2 warp has seen GEMM2 of c - 3 end, so that an evaluating warp polls
+// one barrier per chunk (a poll that succeeds at once takes 100 to 400 cycles
+// beside busy warps): waited for in the middle of chunk c - 1, it also frees
+// the R buffer that chunk c - 1 writes.
+// No waiter falls two phases behind barG1 or four behind the others: all
+// arrivals of barG1 for chunk c + 2 follow barU or barE of c.  A warp reads U of
+// chunk c + 4 only after GEMM1 of c + 4, which is issued after the GEMM1
+// warp's wait for barU of c + 2 and needs W's part of c + 4, issued by the
+// copy warp after its waits for barE of c and barU of c + 1; barG1 of c + 4
+// has the GEMM2 warp's arrival, made after its waits for barE of c + 2 and
+// barG2 of c + 1; GEMM2 of c + 3 needs W's part of c + 3, issued after the copy
+// warp's wait for barG2 of c - 1 and of c.
 // B16 (gradient passes of the BF16 form): GEMM2 takes the single product of
 // R's and W's BF16 high parts (FP32 accumulation) and only R's high part is
 // written to tensor memory; GEMM1, the losses, derivatives and objectives
@@ -391,7 +435,8 @@ dense_pass_kernel(const DenseArgs p, const __grid_constant__ CUtensorMap amap)
 {
     using SM = DnSmem<XSTEP, GRAD, KP>;
     extern __shared__ __align__(1024) unsigned char dsm_dense[];
-    __shared__ uint64_t barA[kDnMaxStages], barP[3], barL[3], barT[3], barG1[2], barG2[2], barU[2], barE[4];
+    __shared__ uint64_t barA[kDnMaxStages], barP[3], barT[3], barG1[2], barG2[4], barU[4], barE[4];
+    __shared__ __align__(16) uint8_t whole_s[4][kDnWarps];  // per chunk (mod 4) and warp: R has no lower parts
     __shared__ uint32_t tslot;
     __shared__ double red[4][kDnRows];
     unsigned char *base = dsm_dense + ((1024 - (smem_u32(dsm_dense) & 1023)) & 1023);
@@ -399,7 +444,7 @@ dense_pass_kernel(const DenseArgs p, const __grid_constant__ CUtensorMap amap)
     unsigned char *fx = base + (size_t)p.nA * SM::a;             // fixed buffers
     unsigned char *pkst = fx;                                    // pk stage s at pkst + s * 3 pk
     unsigned char *ptst = pkst + 9 * SM::pk;                     // pt stage s at ptst + s * 3 pt
-    unsigned char *lsst = ptst + 9 * SM::pt;                     // loss table stage s at lsst + s * ls
+    unsigned char *lsst = ptst + 9 * SM::pt;                     // loss table of A stage s at lsst + s * ls
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int quarter = warp & 3, grp = (warp >> 2) & 3;
@@ -409,8 +454,7 @@ dense_pass_kernel(const DenseArgs p, const __grid_constant__ CUtensorMap amap)
     const int64_t qb = item.q0;
     const int nq = item.nq;
     const int nA = p.nA;
-    // kDnWarps: GEMM1 warp, kDnWarps + 1: copy warp, kDnWarps + 2: GEMM2 warp
-    const bool producer = warp >= kDnWarps;
+    const bool producer = warp >= kDnWarps;  // kDnWarps: GEMM1, kDnWarps + 1: copies, kDnWarps + 2: GEMM2
     // this thread's own row (X-step) or column (Y-step: quarter q of the tile
     // is the 32-column block blocks[4 tile + q]), and its partial slot
     int64_t own = o0 + orow;
@@ -423,18 +467,34 @@ dense_pass_kernel(const DenseArgs p, const __grid_constant__ CUtensorMap amap)
     const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
     const int tb = grp * 16;  // this warp's columns of a chunk
 
-    if (warp == 0) tmem_alloc(&tslot, kDnTmem);
-    if (tid == 0) {
+    // warps 0 .. 3: the own rows, one per thread, on their way while the
+    // barriers and tensor memory are set up
+    float fv[KP];
+    if (grp == 0 && !producer) {
+        const float *f = p.F + own * p.k;
+        if (p.k % 4 == 0 && reinterpret_cast<uintptr_t>(p.F) % 16 == 0) {
+#pragma unroll
+            for (int c = 0; c < KP; c += 4) {
+                const float4 v = (own_ok && c < p.k) ? *reinterpret_cast<const float4 *>(f + c)
+                                                     : make_float4(0.f, 0.f, 0.f, 0.f);
+                fv[c] = v.x;
+                fv[c + 1] = v.y;
+                fv[c + 2] = v.z;
+                fv[c + 3] = v.w;
+            }
+        } else {
+#pragma unroll
+            for (int c = 0; c < KP; ++c) fv[c] = (own_ok && c < p.k) ? f[c] : 0.f;
+        }
+    }
+    if (warp == kDnWarps) tmem_alloc(&tslot, kDnTmem);
+    if (warp == kDnWarps + 1 && lane == 0) {
         for (int s = 0; s < kDnMaxStages; ++s) mbar_init(&barA[s], 1);
         for (int s = 0; s < 3; ++s) mbar_init(&barP[s], 1);
-        for (int s = 0; s < 3; ++s) mbar_init(&barL[s], 1);
         for (int s = 0; s < 3; ++s) mbar_init(&barT[s], 1);
-        mbar_init(&barG1[0], 1);
-        mbar_init(&barG1[1], 1);
-        mbar_init(&barG2[0], 1);
-        mbar_init(&barG2[1], 1);
-        mbar_init(&barU[0], kDnWarps);
-        mbar_init(&barU[1], kDnWarps);
+        for (int s = 0; s < 2; ++s) mbar_init(&barG1[s], 1 + (nA > 2) + (GRAD ? 1 : 0));
+        for (int s = 0; s < 4; ++s) mbar_init(&barG2[s], 1);
+        for (int s = 0; s < 4; ++s) mbar_init(&barU[s], kDnWarps);
         for (int s = 0; s < 4; ++s) mbar_init(&barE[s], kDnWarps);
     }
     // Y-step: this thread's column loss, and whether the warp shares one kind
@@ -445,38 +505,97 @@ dense_pass_kernel(const DenseArgs p, const __grid_constant__ CUtensorMap amap)
     // (a block past the table's last column: lane 0 is inside, the lanes outside
     // take its kind and parameters)
     int wkind = -1;
+    unsigned wkinds = 0;  // the kinds present
     bool wwhole = false;
     if constexpr (!XSTEP) {
         const int k0 = __shfl_sync(0xffffffffu, __float_as_int(myspec.x), 0);
         const float y0 = __shfl_sync(0xffffffffu, myspec.y, 0), z0 = __shfl_sync(0xffffffffu, myspec.z, 0);
         if (!own_ok) myspec = make_float4(__int_as_float(k0), y0, z0, 0.f);
         wkind = __all_sync(0xffffffffu, __float_as_int(myspec.x) == k0) ? k0 : -1;
+        wkinds = __reduce_or_sync(0xffffffffu, 1u << __float_as_int(myspec.x));
         wwhole = __all_sync(0xffffffffu, whole_deriv(__float_as_int(myspec.x), myspec.z));
     }
+
+    bool ok = true;
+    float lacc = 0.f, lcomp = 0.f;
+    // producer bookkeeping (lane 0 of the producer warps)
+    int p_issued = 0, a_issued = 0, t_issued = 0, g1_issued = 0, g2_issued = 0;
+    auto issue_pack = [&](int64_t q) {  // GEMM1's W parts, stage q % 3
+        const int s = (int)((q - qb) % 3);
+        unsigned char *st = pkst + s * 3 * SM::pk;
+        const int64_t t0 = q * kDnNT;
+        mbar_expect_tx(&barP[s], (unsigned)(3 * SM::pk));
+#pragma unroll
+        for (int w = 0; w < 3; ++w)
+            bulk_g2s(st + w * SM::pk, p.pk + w * p.pack_part + t0 * KP, (unsigned)SM::pk, &barP[s]);
+        ++p_issued;
+    };
+    auto issue_pt = [&](int64_t q) {  // GEMM2's W parts, stage q % 3
+        const int s = (int)((q - qb) % 3);
+        unsigned char *st = ptst + s * 3 * SM::pt;
+        mbar_expect_tx(&barT[s], (unsigned)(3 * SM::pt));
+#pragma unroll
+        for (int w = 0; w < 3; ++w)
+            bulk_g2s(st + w * SM::pt, p.pt + w * p.pack_part + q * KP * kDnNT, (unsigned)SM::pt, &barT[s]);
+        ++t_issued;
+    };
+    // Y-step: the tile's 32-column blocks (box q of a stage holds block q)
+    int32_t blk[4] = {-1, -1, -1, -1};
+    unsigned nblk = 0;
+    if (!XSTEP && warp == kDnWarps + 1) {
+        for (int qd = 0; qd < 4; ++qd) {
+            blk[qd] = p.blocks[4 * (int64_t)item.tile + qd];
+            nblk += blk[qd] >= 0 ? 1u : 0u;
+        }
+    }
+    // the A tile (out-of-range elements read as 0) and, X-step, the chunk's
+    // column losses, stage q % nA
+    auto issue_a = [&](int64_t q) {
+        const int s = (int)((q - qb) % nA);
+        unsigned char *dst = ast + s * SM::a;
+        const int t0 = (int)(q * kDnNT);
+        if constexpr (XSTEP) {
+            const int nv = (int)(p.nother - t0 < kDnNT ? p.nother - t0 : kDnNT);
+            mbar_expect_tx(&barA[s], (unsigned)(SM::a + nv * sizeof(LossF)));
+            tma_load_2d(dst, &amap, t0, (int)o0, &barA[s]);
+            tma_load_2d(dst + SM::a / 2, &amap, t0 + 32, (int)o0, &barA[s]);
+            bulk_g2s(lsst + s * SM::ls, p.lossf + t0, (unsigned)(nv * sizeof(LossF)), &barA[s]);
+        } else {
+            mbar_expect_tx(&barA[s], nblk * (unsigned)(SM::a / 4));
+            for (int qd = 0; qd < 4; ++qd)
+                if (blk[qd] >= 0) tma_load_2d(dst + qd * (SM::a / 4), &amap, 32 * blk[qd], t0, &barA[s]);
+        }
+        ++a_issued;
+    };
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t taddr = tslot;
+    // the first copies start while the own rows are written to tensor memory
+    if (warp == kDnWarps + 1 && elect_one()) {
+        for (int s = 0; s < 3 && s < nq; ++s) issue_pack(qb + s);
+        for (int s = 0; s < nA && s < nq; ++s) issue_a(qb + s);
+        if (GRAD)
+            for (int s = 0; s < 2 && s < nq; ++s) issue_pt(qb + s);
+    }
     // own rows split in three into tensor memory (GEMM1's A operand, two BF16
-    // values per column along k): warps 0 .. 3, one row per thread
+    // values per column along k)
     if (grp == 0 && !producer) {
 #pragma unroll
         for (int c0 = 0; c0 < KP; c0 += 16) {
             uint32_t hv[8], mv[8], lv[8];
 #pragma unroll
             for (int w = 0; w < 16; w += 2) {
-                const float v0 = (own_ok && c0 + w < p.k) ? p.F[own * p.k + c0 + w] : 0.f;
-                const float v1 = (own_ok && c0 + w + 1 < p.k) ? p.F[own * p.k + c0 + w + 1] : 0.f;
                 __nv_bfloat16 h0, m0, l0, h1, m1, l1;
-                split3(v0, h0, m0, l0);
-                split3(v1, h1, m1, l1);
+                split3(fv[c0 + w], h0, m0, l0);
+                split3(fv[c0 + w + 1], h1, m1, l1);
                 hv[w / 2] = bf2_bits(__halves2bfloat162(h0, h1));
                 mv[w / 2] = bf2_bits(__halves2bfloat162(m0, m1));
                 lv[w / 2] = bf2_bits(__halves2bfloat162(l0, l1));
             }
-            tmem_st8(taddr + lane_base + (uint32_t)(kDnColOwn + c0 / 2), hv);
-            tmem_st8(taddr + lane_base + (uint32_t)(kDnColOwn + KP / 2 + c0 / 2), mv);
-            tmem_st8(taddr + lane_base + (uint32_t)(kDnColOwn + KP + c0 / 2), lv);
+            tmem_st8(taddr + lane_base + (uint32_t)(DnG<KP>::Own + c0 / 2), hv);
+            tmem_st8(taddr + lane_base + (uint32_t)(DnG<KP>::Own + KP / 2 + c0 / 2), mv);
+            tmem_st8(taddr + lane_base + (uint32_t)(DnG<KP>::Own + KP + c0 / 2), lv);
         }
         tmem_wait_st();
     }
@@ -484,217 +603,161 @@ dense_pass_kernel(const DenseArgs p, const __grid_constant__ CUtensorMap amap)
     __syncthreads();
     tc_fence_after();
 
-    bool ok = true;
-    float lacc = 0.f, lcomp = 0.f;
-    // producer bookkeeping (warp kDnWarps, lane 0)
-    int p_issued = 0, a_issued = 0, t_issued = 0, l_issued = 0, g1_issued = 0, g2_issued = 0;
     if (producer) {
-        if (lane == 0) {
-            auto issue_pack = [&](int64_t q) {  // GEMM1's W parts, stage q % 3
-                const int s = (int)((q - qb) % 3);
-                unsigned char *st = pkst + s * 3 * SM::pk;
-                const int64_t t0 = q * kDnNT;
-                mbar_expect_tx(&barP[s], (unsigned)(3 * SM::pk));
-#pragma unroll
-                for (int w = 0; w < 3; ++w)
-                    bulk_g2s(st + w * SM::pk, p.pk + w * p.pack_part + t0 * KP, (unsigned)SM::pk, &barP[s]);
-                ++p_issued;
-            };
-            auto issue_ls = [&](int64_t q) {  // X-step: the chunk's column losses, stage q % 3
-                const int s = (int)((q - qb) % 3);
-                const int64_t t0 = q * kDnNT;
-                const int nv = (int)(p.nother - t0 < kDnNT ? p.nother - t0 : kDnNT);
-                mbar_expect_tx(&barL[s], (unsigned)(nv * sizeof(LossF)));
-                bulk_g2s(lsst + s * SM::ls, p.lossf + t0, (unsigned)(nv * sizeof(LossF)), &barL[s]);
-                ++l_issued;
-            };
-            auto issue_pt = [&](int64_t q) {  // GEMM2's W parts, stage q % 3
-                const int s = (int)((q - qb) % 3);
-                unsigned char *st = ptst + s * 3 * SM::pt;
-                mbar_expect_tx(&barT[s], (unsigned)(3 * SM::pt));
-#pragma unroll
-                for (int w = 0; w < 3; ++w)
-                    bulk_g2s(st + w * SM::pt, p.pt + w * p.pack_part + q * KP * kDnNT, (unsigned)SM::pt, &barT[s]);
-                ++t_issued;
-            };
-            // Y-step: the tile's 32-column blocks (box q of a stage holds block q)
-            int32_t blk[4] = {-1, -1, -1, -1};
-            unsigned nblk = 0;
-            if constexpr (!XSTEP) {
-                for (int qd = 0; qd < 4; ++qd) {
-                    blk[qd] = p.blocks[4 * (int64_t)item.tile + qd];
-                    nblk += blk[qd] >= 0 ? 1u : 0u;
-                }
-            }
-            auto issue_a = [&](int64_t q) {  // the A tile, stage q % nA (out-of-range elements read as 0)
-                const int s = (int)((q - qb) % nA);
-                unsigned char *dst = ast + s * SM::a;
-                const int t0 = (int)(q * kDnNT);
-                if constexpr (XSTEP) {
-                    mbar_expect_tx(&barA[s], (unsigned)SM::a);
-                    tma_load_2d(dst, &amap, t0, (int)o0, &barA[s]);
-                    tma_load_2d(dst + SM::a / 2, &amap, t0 + 32, (int)o0, &barA[s]);
-                } else {
-                    mbar_expect_tx(&barA[s], nblk * (unsigned)(SM::a / 4));
-                    for (int qd = 0; qd < 4; ++qd)
-                        if (blk[qd] >= 0) tma_load_2d(dst + qd * (SM::a / 4), &amap, 32 * blk[qd], t0, &barA[s]);
-                }
-                ++a_issued;
-            };
-            // GEMM1 of chunk q into accumulator buffer (q - qb) % 2, once its W parts are in
-            auto issue_gemm1 = [&](int64_t q) -> bool {
-                const int c = (int)(q - qb);
+        const bool lead = elect_one();  // the lane that issues
+        if (warp == kDnWarps && lead) {
+            // GEMM1 warp.  (own part, W part), smallest products first; hi . hi last
+            constexpr int pa[6] = {1, 0, 2, 0, 1, 0};
+            constexpr int pb[6] = {1, 2, 0, 1, 0, 0};
+            for (int c = 0; ok && c < nq; ++c) {
                 const int s = c % 3, b = c & 1;
-                if (!mbar_wait_bounded(&barP[s], (unsigned)(c / 3) & 1u)) return false;
+                // U of chunk c - 2 is in registers, W's parts of chunk c are in
+                if (c > 1) ok = mbar_wait_bounded(&barU[(c - 2) & 3], (unsigned)((c - 2) >> 2) & 1u);
+                ok = ok && mbar_wait_bounded(&barP[s], (unsigned)(c / 3) & 1u);
+                if (!ok) break;
                 tc_fence_after();
-                const uint32_t idesc = umma_idesc_bf16(kDnRows, kDnNT);
-                const unsigned char *w = pkst + s * 3 * SM::pk;
+                constexpr uint32_t idesc = umma_idesc_bf16(kDnRows, kDnNT);
                 constexpr uint32_t RB = 2 * KP;  // bytes per W row; a K step of 16 is 32 bytes, 8 own columns
-                // (own part, W part), smallest products first; hi . hi last
-                const int pa[6] = {1, 0, 2, 0, 1, 0};
-                const int pb[6] = {1, 2, 0, 1, 0, 0};
+                const uint64_t d0 = umma_desc_sw(pkst + s * 3 * SM::pk, RB);
 #pragma unroll
                 for (int pr = 0; pr < 6; ++pr)
 #pragma unroll
                     for (int ks = 0; ks < KP / 16; ++ks)
                         umma_bf16_ta(taddr + (uint32_t)(b * kDnNT),
-                                     taddr + (uint32_t)(kDnColOwn + pa[pr] * (KP / 2) + ks * 8),
-                                     umma_desc_sw(w + pb[pr] * SM::pk + ks * 32, RB), idesc, pr > 0 || ks > 0);
+                                     taddr + (uint32_t)(DnG<KP>::Own + pa[pr] * (KP / 2) + ks * 8),
+                                     d0 + ((pb[pr] * SM::pk + ks * 32) >> 4), idesc, pr > 0 || ks > 0);
                 umma_commit(&barG1[b]);
                 ++g1_issued;
-                return true;
-            };
-            // GEMM2 of chunk q: G += R W, R from tensor memory
-            auto issue_gemm2 = [&](int64_t q) -> bool {
-                const int c = (int)(q - qb);
-                const int s = c % 3, rb = c & 1;
-                if (!mbar_wait_bounded(&barT[s], (unsigned)(c / 3) & 1u)) return false;
+            }
+        } else if (GRAD && warp == kDnWarps + 2 && lead) {
+            // GEMM2 warp: G += R W, R from tensor memory (a K = 16 step of R is 8 columns)
+            mbar_arrive(&barG1[0]);
+            if (nq > 1) mbar_arrive(&barG1[1]);
+            for (int c = 0; ok && c < nq; ++c) {
+                const int s = c % 3;
+                ok = mbar_wait_bounded(&barT[s], (unsigned)(c / 3) & 1u);
+                ok = ok && mbar_wait_bounded(&barE[c & 3], (unsigned)(c >> 2) & 1u);  // R of chunk c is written
+                // GEMM2 of c - 1 is done: chunk c + 1 may write its R buffer once
+                // the warps have seen barG1 of c + 2
+                if (c > 0) ok = ok && mbar_wait_bounded(&barG2[(c - 1) & 3], (unsigned)((c - 1) >> 2) & 1u);
+                if (!ok) break;
+                if (c + 2 < nq) mbar_arrive(&barG1[c & 1]);
                 tc_fence_after();
-                const uint32_t idesc = umma_idesc_bf16(kDnRows, KP);
-                const unsigned char *wt = ptst + s * 3 * SM::pt;
-                // (R part, W part), smallest products first; a K = 16 step of R is 8 columns
-                const int pa[6] = {1, 0, 2, 0, 1, 0};
-                const int pb[6] = {1, 2, 0, 1, 0, 0};
-                constexpr int P0 = B16 ? 5 : 0;  // the BF16 form: hi . hi only
+                const uint64_t d0 = umma_desc_sw(ptst + s * 3 * SM::pt, 2 * kDnNT);
+                const uint32_t r0 = taddr + (uint32_t)(kDnColR + (c & 1) * 96);
+                // the four warps of each 16 chunk columns say whether R has lower parts there
+                uint32_t wh[4];
+                *reinterpret_cast<uint4 *>(wh) = *reinterpret_cast<const uint4 *>(whole_s[c & 3]);
 #pragma unroll
-                for (int pr = P0; pr < 6; ++pr)
-#pragma unroll
-                    for (int ks = 0; ks < kDnNT / 16; ++ks)
-                        umma_bf16_ta(taddr + kDnColG, taddr + (uint32_t)(kDnColR + rb * 96 + pa[pr] * 32 + ks * 8),
-                                     umma_desc_sw(wt + pb[pr] * SM::pt + ks * 32, 2 * kDnNT), idesc,
-                                     c > 0 || pr > P0 || ks > 0);
-                umma_commit(&barG2[rb]);
+                for (int ks = 0; ks < kDnNT / 16; ++ks) {
+                    const uint64_t dk = d0 + ((ks * 32) >> 4);
+                    const uint32_t rk = r0 + ks * 8;
+                    if constexpr (B16) {  // the BF16 form: hi . hi only
+                        umma_bf16_ta(taddr + kDnColG, rk, dk, umma_idesc_bf16(kDnRows, KP), c > 0 || ks > 0);
+                    } else if constexpr (DnG<KP>::NB == 3) {
+                        umma_bf16_ta(taddr + kDnColG, rk, dk, umma_idesc_bf16(kDnRows, 3 * KP), c > 0 || ks > 0);
+                        if (wh[ks] != 0x01010101u) {
+                            umma_bf16_ta(taddr + kDnColG, rk + 32, dk, umma_idesc_bf16(kDnRows, 2 * KP), true);
+                            umma_bf16_ta(taddr + kDnColG, rk + 64, dk, umma_idesc_bf16(kDnRows, KP), true);
+                        }
+                    } else {
+                        constexpr uint32_t id = umma_idesc_bf16(kDnRows, KP);
+                        umma_bf16_ta(taddr + kDnColG, rk, dk + (2 * SM::pt >> 4), id, c > 0 || ks > 0);
+                        if (wh[ks] != 0x01010101u) {
+                            umma_bf16_ta(taddr + kDnColG, rk + 32, dk + (SM::pt >> 4), id, true);
+                            umma_bf16_ta(taddr + kDnColG, rk + 64, dk, id, true);
+                            umma_bf16_ta(taddr + kDnColG, rk + 32, dk, id, true);
+                        }
+                        umma_bf16_ta(taddr + kDnColG, rk, dk + (SM::pt >> 4), id, true);
+                        umma_bf16_ta(taddr + kDnColG, rk, dk, id, true);
+                    }
+                }
+                umma_commit(&barG2[c & 3]);
                 ++g2_issued;
-                return true;
-            };
-            if (warp == kDnWarps) {
-                // GEMM1 warp: W's GEMM1 parts and GEMM1
-                for (int s = 0; s < 3 && s < nq; ++s) issue_pack(qb + s);
-                ok = issue_gemm1(qb);
-                if (ok && nq > 1) ok = issue_gemm1(qb + 1);
-                for (int it = 0; ok && it < nq; ++it) {
-                    const int64_t q = qb + it;
-                    // U of chunk q has been read (so GEMM1 of q is done): its
-                    // accumulator buffer takes chunk q + 2, its W stage chunk q + 3
-                    if (!mbar_wait_bounded(&barU[it & 1], (unsigned)(it >> 1) & 1u)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    if (it + 3 < nq) issue_pack(q + 3);
-                    if (it + 2 < nq && !issue_gemm1(q + 2)) {
-                        ok = false;
-                        break;
-                    }
+            }
+        } else if (warp == kDnWarps + 1 && lead) {
+            for (int c = 0; ok && nA > 2 && c < 2 && c < nq; ++c) {
+                ok = mbar_wait_bounded(&barA[c], 0);
+                if (ok) mbar_arrive(&barG1[c]);
+            }
+            for (int it = 0; ok && it < nq; ++it) {
+                const int64_t q = qb + it;
+                // U of chunk it is read, so GEMM1 of it has read its W stage
+                ok = mbar_wait_bounded(&barU[it & 3], (unsigned)(it >> 2) & 1u);
+                if (!ok) break;
+                if (it + 3 < nq) issue_pack(q + 3);
+                if (nA > 2 && it + 2 < nq) {  // barG1's arrival for the A tile of it + 2
+                    ok = mbar_wait_bounded(&barA[(it + 2) % nA], (unsigned)((it + 2) / nA) & 1u);
+                    if (!ok) break;
+                    mbar_arrive(&barG1[it & 1]);
                 }
-            } else if (warp == kDnWarps + 2) {
-                // GEMM2 warp (gradient passes): G += R W once R of chunk q is written
-                for (int it = 0; GRAD && it < nq; ++it) {
-                    if (!mbar_wait_bounded(&barE[it & 3], (unsigned)(it >> 2) & 1u)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    if (!issue_gemm2(qb + it)) {
-                        ok = false;
-                        break;
-                    }
-                }
-            } else {
-                // copy warp: A tiles, loss tables and W's GEMM2 parts
-                for (int s = 0; s < nA && s < nq; ++s) issue_a(qb + s);
-                if (XSTEP)
-                    for (int s = 0; s < 3 && s < nq; ++s) issue_ls(qb + s);
-                if (GRAD) {
-                    issue_pt(qb);
-                    if (nq > 1) issue_pt(qb + 1);
-                }
-                for (int it = 0; it < nq; ++it) {
-                    const int64_t q = qb + it;
-                    // the entries of chunk q are done: its A stage and loss-table
-                    // stage are free, and (the warps having waited for GEMM2 of
-                    // q - 2 before writing R of q) so is the GEMM2 stage of q - 2
-                    if (!mbar_wait_bounded(&barE[it & 3], (unsigned)(it >> 2) & 1u)) {
-                        ok = false;
-                        break;
-                    }
-                    if (it + nA < nq) issue_a(q + nA);
-                    if (XSTEP && it + 3 < nq) issue_ls(q + 3);
-                    if (GRAD && it >= 1 && it + 1 < nq) issue_pt(q + 1);
+                // the entries of chunk it are done: its A stage is free
+                ok = mbar_wait_bounded(&barE[it & 3], (unsigned)(it >> 2) & 1u);
+                if (!ok) break;
+                if (it + nA < nq) issue_a(q + nA);
+                if (GRAD && it + 2 < nq) {
+                    // GEMM2 of it - 1 leaves the stage of it + 2
+                    if (it > 0) ok = mbar_wait_bounded(&barG2[(it - 1) & 3], (unsigned)((it - 1) >> 2) & 1u);
+                    if (ok) issue_pt(q + 2);
                 }
             }
         }
     } else {
-        // ring positions and phases of the A and loss-table stages, kept as
-        // counters (a chunk is about 250 instructions of a warp: a division
-        // by the stage count would be a tenth of them)
-        int sA = 0, sL = 0;
-        unsigned phA = 0, phL = 0;
+        int sA = 0;  // ring position of the A stage, a counter (a chunk is few hundred instructions: no division)
         const bool own_all = __all_sync(0xffffffffu, own_ok), own_any = __any_sync(0xffffffffu, own_ok);
         int64_t left = p.nother - qb * kDnNT - tb;  // entries of the other dimension from this warp's first on
-        for (int it = 0; it < nq; ++it, left -= kDnNT) {
-            const int b = it & 1;
-            // the A tile (and the loss table) lands chunks ahead: its values
-            // are read before the wait for U
-            if (XSTEP) ok = ok && mbar_wait_bounded(&barL[sL], phL);
-            ok = ok && mbar_wait_bounded(&barA[sA], phA);
+        float u[16], a[16];
+        uint32_t ur[16];
+        // this warp's cells of the A stage sA
+        auto load_a = [&]() {
+            const unsigned char *as = ast + sA * SM::a;
+            if constexpr (XSTEP) {
+                // box tb / 32, row orow: 16-byte units (tb % 32) / 4 .. + 3, swizzled
+                const unsigned char *row = as + (tb >> 5) * (SM::a / 2) + orow * 128;
+#pragma unroll
+                for (int w = 0; w < 4; ++w) {
+                    const float4 v =
+                        *reinterpret_cast<const float4 *>(row + ((((tb & 31) >> 2) + w) ^ (orow & 7)) * 16);
+                    a[4 * w] = v.x;
+                    a[4 * w + 1] = v.y;
+                    a[4 * w + 2] = v.z;
+                    a[4 * w + 3] = v.w;
+                }
+            } else {
+                // box `quarter`: 64 chunk rows x 32 columns
+                const float *af = reinterpret_cast<const float *>(as) + quarter * (kDnNT * 32);
+#pragma unroll
+                for (int w = 0; w < 16; ++w) a[w] = af[(tb + w) * 32 + lane];
+            }
+        };
+        // wait for U and A of chunk c (stage sA) and start loading both; whole
+        // warp, false when the wait ran out
+        auto start_loads = [&](int c) -> bool {
+            bool w = mbar_wait_bounded(&barG1[c & 1], (unsigned)(c >> 1) & 1u);
+            if (nA == 2) w = w && mbar_wait_bounded(&barA[sA], (unsigned)(c >> 1) & 1u);
+            tc_fence_after();
+            w = __all_sync(0xffffffffu, w);  // tcgen05.ld / st are warp-collective
+            if (w) {
+                tmem_ld16_start(taddr + lane_base + (uint32_t)((c & 1) * kDnNT + tb), ur);
+                load_a();
+            }
+            return w;
+        };
+        ok = start_loads(0);
+        for (int it = 0; ok && it < nq; ++it, left -= kDnNT) {
+            tmem_ld16_wait(ur, u);
+            // U of this chunk is in registers: its accumulator may take GEMM1 of it + 2
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&barU[it & 3]);
             float lsum = 0.f;
             float rr[16];
             bool whole = false;  // every derivative is a whole number BF16 holds
             {
-                const unsigned char *as = ast + sA * SM::a;
-                float u[16], a[16];
-                if constexpr (XSTEP) {
-                    // box tb / 32, row orow: 16-byte units (tb % 32) / 4 .. + 3, swizzled
-                    const unsigned char *row = as + (tb >> 5) * (SM::a / 2) + orow * 128;
-#pragma unroll
-                    for (int w = 0; w < 4; ++w) {
-                        const float4 v =
-                            *reinterpret_cast<const float4 *>(row + ((((tb & 31) >> 2) + w) ^ (orow & 7)) * 16);
-                        a[4 * w] = v.x;
-                        a[4 * w + 1] = v.y;
-                        a[4 * w + 2] = v.z;
-                        a[4 * w + 3] = v.w;
-                    }
-                } else {
-                    // box `quarter`: 64 chunk rows x 32 columns
-                    const float *af = reinterpret_cast<const float *>(as) + quarter * (kDnNT * 32);
-#pragma unroll
-                    for (int w = 0; w < 16; ++w) a[w] = af[(tb + w) * 32 + lane];
-                }
-                ok = ok && mbar_wait_bounded(&barG1[b], (unsigned)(it >> 1) & 1u);
-                tc_fence_after();
-                ok = __all_sync(0xffffffffu, ok);  // tcgen05.ld / st below are warp-collective
-                if (!ok) break;
-                tmem_ld16(taddr + lane_base + (uint32_t)(b * kDnNT + tb), u);
-                // U of this chunk is in registers: its buffer may take the next GEMM1
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&barU[b]);
                 const bool full = own_all && left >= 16;
                 const uint32_t valid =
                     !own_ok ? 0u : (left >= 16 ? 0xffffu : (left <= 0 ? 0u : (1u << left) - 1u));
-                const LossF *lf = reinterpret_cast<const LossF *>(lsst + sL * SM::ls) + tb;
+                const LossF *lf = reinterpret_cast<const LossF *>(lsst + sA * SM::ls) + tb;
                 // the kind (and parameters) the 16 entries share, -1 if they do not:
                 // X-step, kept in the w of each column's loss; Y-step, the warp's columns
                 int kind = wkind;
@@ -712,8 +775,8 @@ dense_pass_kernel(const DenseArgs p, const __grid_constant__ CUtensorMap amap)
 #pragma unroll
                     for (int w = 0; w < 16; ++w) rr[w] = 0.f;
                     whole = true;
-                } else if (kind < 0) {
-                    dn_block_any<XSTEP>(u, a, lf, myspec, valid, rr, lsum);
+                } else if (XSTEP && kind < 0) {
+                    dn_block_any(u, a, lf, valid, rr, lsum);
                 } else {
                     whole = !WGT && (XSTEP ? whole_deriv(kind, lev) : wwhole);
                     if (!full) {  // cells outside the table count as missing
@@ -721,23 +784,17 @@ dense_pass_kernel(const DenseArgs p, const __grid_constant__ CUtensorMap amap)
                         for (int w = 0; w < 16; ++w)
                             if (!((valid >> w) & 1u)) a[w] = __int_as_float(0x7fffffff);
                     }
-                    if (MISS || !full) {
-                        switch (kind) {
-                        case kLossQuad: dn_block<kLossQuad, true>(u, a, prm, lev, rr, lsum); break;
-                        case kLossHuber: dn_block<kLossHuber, true>(u, a, prm, lev, rr, lsum); break;
-                        case kLossHinge: dn_block<kLossHinge, true>(u, a, prm, lev, rr, lsum); break;
-                        case kLossLogistic: dn_block<kLossLogistic, true>(u, a, prm, lev, rr, lsum); break;
-                        case kLossOrdinal: dn_block<kLossOrdinal, true>(u, a, prm, lev, rr, lsum); break;
-                        default: dn_block_any<XSTEP>(u, a, lf, myspec, valid, rr, lsum); break;
-                        }
+                    if (!MISS && full && kind >= 0) {
+                        dn_block_kind<false>(kind, u, a, prm, lev, rr, lsum);
+                    } else if (XSTEP || kind >= 0) {
+                        dn_block_kind<true>(kind, u, a, prm, lev, rr, lsum);
                     } else {
-                        switch (kind) {
-                        case kLossQuad: dn_block<kLossQuad, false>(u, a, prm, lev, rr, lsum); break;
-                        case kLossHuber: dn_block<kLossHuber, false>(u, a, prm, lev, rr, lsum); break;
-                        case kLossHinge: dn_block<kLossHinge, false>(u, a, prm, lev, rr, lsum); break;
-                        case kLossLogistic: dn_block<kLossLogistic, false>(u, a, prm, lev, rr, lsum); break;
-                        case kLossOrdinal: dn_block<kLossOrdinal, false>(u, a, prm, lev, rr, lsum); break;
-                        default: dn_block_any<XSTEP>(u, a, lf, myspec, valid, rr, lsum); break;
+                        // Y-step, a 32-column block that mixes kinds: kind by
+                        // kind, the lanes of that kind
+                        for (unsigned todo = wkinds; todo; todo &= todo - 1u) {
+                            const int kd = __ffs((int)todo) - 1;
+                            if (kd == __float_as_int(myspec.x)) dn_block_kind<true>(kd, u, a, prm, lev, rr, lsum);
+                            __syncwarp();
                         }
                     }
                 }
@@ -747,6 +804,15 @@ dense_pass_kernel(const DenseArgs p, const __grid_constant__ CUtensorMap amap)
                     for (int w = 0; w < 16; ++w) rr[w] *= wown;
                 }
             }
+            // the next chunk's loads start here
+            if (++sA == nA) sA = 0;
+            if (it + 1 < nq) ok = start_loads(it + 1);
+            else if (GRAD && nq > 2) {  // (no later U to wait for)
+                ok = mbar_wait_bounded(&barG2[(nq - 3) & 3], (unsigned)((nq - 3) >> 2) & 1u);
+                tc_fence_after();
+                ok = __all_sync(0xffffffffu, ok);
+            }
+            if (!ok) break;
             // compensated FP32 running sum of the chunk sums
             {
                 const float y = lsum - lcomp;
@@ -755,12 +821,6 @@ dense_pass_kernel(const DenseArgs p, const __grid_constant__ CUtensorMap amap)
                 lacc = t;
             }
             if constexpr (GRAD) {
-                // R of the previous chunk is no longer read once its GEMM2 is done
-                // R buffer it % 2 is free once GEMM2 of it - 2 is done
-                if (it > 1) ok = mbar_wait_bounded(&barG2[b], (unsigned)((it - 2) >> 1) & 1u);
-                tc_fence_after();
-                ok = __all_sync(0xffffffffu, ok);
-                if (!ok) break;
                 uint32_t hi[8], mi[8], lo[8];
                 const unsigned long long m1 = pk2(-1.f, -1.f);
                 if (B16 || whole) {  // (whole: warp-uniform) the high parts are all of R
@@ -787,7 +847,7 @@ dense_pass_kernel(const DenseArgs p, const __grid_constant__ CUtensorMap amap)
                         lo[w / 2] = bf2_bits(__floats2bfloat162_rn(b0, b1));
                     }
                 }
-                const uint32_t rcol = kDnColR + (uint32_t)(b * 96 + tb / 2);
+                const uint32_t rcol = kDnColR + (uint32_t)((it & 1) * 96 + tb / 2);
                 tmem_st8(taddr + lane_base + rcol, hi);
                 if constexpr (!B16) {
                     tmem_st8(taddr + lane_base + rcol + 32, mi);
@@ -797,19 +857,13 @@ dense_pass_kernel(const DenseArgs p, const __grid_constant__ CUtensorMap amap)
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&barE[it & 3]);
-            if (++sA == nA) {
-                sA = 0;
-                phA ^= 1u;
-            }
-            if (XSTEP && ++sL == 3) {
-                sL = 0;
-                phL ^= 1u;
+            if (lane == 0) {
+                if (GRAD) whole_s[it & 3][4 * grp + quarter] = whole ? 1 : 0;
+                mbar_arrive(&barE[it & 3]);
             }
         }
         if (GRAD && ok) {
-            ok = mbar_wait_bounded(&barG2[(nq - 1) & 1], (unsigned)((nq - 1) >> 1) & 1u);
-            if (ok && nq > 1) ok = mbar_wait_bounded(&barG2[nq & 1], (unsigned)((nq - 2) >> 1) & 1u);
+            ok = mbar_wait_bounded(&barG2[(nq - 1) & 3], (unsigned)((nq - 1) >> 2) & 1u);
             tc_fence_after();
             ok = __all_sync(0xffffffffu, ok);
         }
@@ -823,6 +877,13 @@ dense_pass_kernel(const DenseArgs p, const __grid_constant__ CUtensorMap amap)
             for (int bb = 0; bb < KP / 16; ++bb) {
                 float v[16];
                 tmem_ld16(taddr + lane_base + (uint32_t)(kDnColG + 16 * bb), v);
+                if constexpr (DnG<KP>::NB == 3 && !B16) {  // the products with W's mid and lo parts
+                    float v1[16], v2[16];
+                    tmem_ld16(taddr + lane_base + (uint32_t)(kDnColG + KP + 16 * bb), v1);
+                    tmem_ld16(taddr + lane_base + (uint32_t)(kDnColG + 2 * KP + 16 * bb), v2);
+#pragma unroll
+                    for (int w = 0; w < 16; ++w) v[w] += v1[w] + v2[w];
+                }
                 if (own_ok) {
 #pragma unroll
                     for (int w = 0; w < 16; ++w)
@@ -834,14 +895,12 @@ dense_pass_kernel(const DenseArgs p, const __grid_constant__ CUtensorMap amap)
     __syncthreads();
     if (!fail && !producer && grp == 0 && own_ok)
         p.part_loss[slot] = red[0][orow] + red[1][orow] + red[2][orow] + red[3][orow];
-    if (fail && producer && lane == 0) {  // each producer warp drains what it issued
+    if (fail && producer && elect_one()) {  // each producer warp drains what it issued (the same lane as above)
         atomicOr(p.err, 1);
         // wait (bounded) for the last copy into each stage and the last MMA
         // batches: every earlier one completed before a later one was issued
         for (int c = p_issued - 3 > 0 ? p_issued - 3 : 0; c < p_issued; ++c)
             mbar_wait_bounded(&barP[c % 3], (unsigned)(c / 3) & 1u);
-        for (int c = l_issued - 3 > 0 ? l_issued - 3 : 0; c < l_issued; ++c)
-            mbar_wait_bounded(&barL[c % 3], (unsigned)(c / 3) & 1u);
         for (int c = a_issued - nA > 0 ? a_issued - nA : 0; c < a_issued; ++c)
             mbar_wait_bounded(&barA[c % nA], (unsigned)(c / nA) & 1u);
         for (int c = t_issued - 3 > 0 ? t_issued - 3 : 0; c < t_issued; ++c)
@@ -849,11 +908,11 @@ dense_pass_kernel(const DenseArgs p, const __grid_constant__ CUtensorMap amap)
         for (int c = g1_issued - 2 > 0 ? g1_issued - 2 : 0; c < g1_issued; ++c)
             mbar_wait_bounded(&barG1[c & 1], (unsigned)(c >> 1) & 1u);
         for (int c = g2_issued - 2 > 0 ? g2_issued - 2 : 0; c < g2_issued; ++c)
-            mbar_wait_bounded(&barG2[c & 1], (unsigned)(c >> 1) & 1u);
+            mbar_wait_bounded(&barG2[c & 3], (unsigned)(c >> 2) & 1u);
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 0) {
+    if (warp == kDnWarps) {
         tc_fence_after();
         tmem_dealloc(taddr, kDnTmem);
     }
