@@ -5,12 +5,15 @@
 // every segment s (row in the X-step, column in the Y-step),
 //     (sum_{e in s} w_e w_e^T + gamma I) f_s = sum_{e in s} a_e w_e.
 // Launch 1 (per chunk): partial Gram lower triangle and right-hand side in
-// the element type.  Launch 2 (per segment, one warp): sum of the partials in
-// a fixed order, then an FP64 Cholesky factorisation and two triangular
-// solves in shared memory.
+// the element type.  Launch 2 (per segment): sum of the partials in a fixed
+// order, then the solve: FP64 models (and prox-prox) an FP64 Cholesky
+// factorisation and two triangular solves in shared memory, one warp per
+// segment; FP32 models the refined solve of glrm_spd.cuh, K lanes per segment,
+// with the FP64 factorisation for the systems it does not settle.
 #pragma once
 
 #include "glrm_engine.cuh"
+#include "glrm_spd.cuh"
 
 namespace glrm {
 
@@ -32,50 +35,105 @@ __device__ __forceinline__ void tri_rc(int p, int &r, int &c)
     c = p - r * (r + 1) / 2;
 }
 
+// One warp per chunk.  Rows of the other factor come in batches of kRows
+// through two shared-memory buffers filled by cp.async (16-byte pieces when
+// the rows allow it: eight lanes fetch one 128-byte row, where a lane per row
+// touched 32 lines with every load); the 32 / K lane groups take the batch's
+// entries in turn, each accumulating its whole K x K tile in registers
+// (GramTile), and are summed at the end.  On the 100,000 x 20,000 completion
+// table (k = 32, 2e7 entries) 4.5 -> 0.94 (rows) and 4.7 -> 1.02 ms (columns); bound by the FP32
+// multiply-adds of the full square (1,024 per entry).
 template <class T, int K>
 __global__ void __launch_bounds__(kAlsWarps * 32)
 als_gram_kernel(int64_t nchunks, const int4 *__restrict__ chunks, const int32_t *__restrict__ idx,
-                const T *__restrict__ val, const T *__restrict__ W, int k, T *__restrict__ part)
+                const T *__restrict__ val, const T *__restrict__ W, int k, bool vec, T *__restrict__ part)
 {
     using TR = Tri<K>;
-    __shared__ T wsh[kAlsWarps][32][K + 1];
-    __shared__ T ash[kAlsWarps][32];
+    using GT = GramTile<T, K>;
+    constexpr int kRows = sizeof(T) == 4 ? 32 : 16;   // entries per batch
+    constexpr int GR = 32 / K;                        // lane groups
+    constexpr int PPR = K * (int)sizeof(T) / 16;      // 16-byte pieces per row
+    __shared__ __align__(16) T wsh[kAlsWarps][2][kRows][K];
+    __shared__ T ash[kAlsWarps][2][kRows];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int64_t c = (int64_t)blockIdx.x * kAlsWarps + wid;
     if (c >= nchunks) return;
     const int4 ch = chunks[c];
-    int rq[TR::NP], cq[TR::NP];
-    T acc[TR::NP];
+    // coordinates from k to K are zero and stay so
+    for (int q = lane; q < 2 * kRows * K; q += 32) (&wsh[wid][0][0][0])[q] = T(0);
+    __syncwarp();
+    GT g;
+    g.init(lane % K);
+    int j = 0;
+    T a = T(0);
+    auto fetch = [&](int base) {  // index and value of entry base + lane
+        if (lane < kRows && base + lane < ch.z) {
+            j = __ldg(idx + base + lane);
+            a = __ldg(val + base + lane);
+        }
+    };
+    auto issue = [&](int buf, int base) {  // the fetched batch's rows into a buffer
+        const int cnt = min(kRows, ch.z - base);
+        if (vec) {
 #pragma unroll
-    for (int q = 0; q < TR::NP; ++q) {
-        const int p = lane + 32 * q;
-        tri_rc(p < TR::N ? p : 0, rq[q], cq[q]);
-        acc[q] = T(0);
-    }
-    T bacc = T(0);
-    for (int base = ch.y; base < ch.z; base += 32) {
-        const int e = base + lane;
-        if (e < ch.z) {
-            const int64_t j = __ldg(idx + e);
-            ash[wid][lane] = __ldg(val + e);
-#pragma unroll
-            for (int q = 0; q < K; ++q) wsh[wid][lane][q] = q < k ? __ldg(W + j * k + q) : T(0);
+            for (int q = 0; q < kRows * PPR / 32; ++q) {
+                const int row = (q * 32 + lane) / PPR, piece = (q * 32 + lane) % PPR;
+                const int jr = __shfl_sync(0xffffffffu, j, row);
+                if (row < cnt && piece * (16 / (int)sizeof(T)) < k)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                                     smem_u32(&wsh[wid][buf][row][piece * (16 / (int)sizeof(T))])),
+                                 "l"(W + (int64_t)jr * k + piece * (16 / (int)sizeof(T)))
+                                 : "memory");
+            }
+        } else {
+            for (int e = 0; e < cnt; ++e) {
+                const int jr = __shfl_sync(0xffffffffu, j, e);
+                if (lane < k)
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_u32(&wsh[wid][buf][e][lane])),
+                                 "l"(W + (int64_t)jr * k + lane), "n"((int)sizeof(T))
+                                 : "memory");
+            }
+        }
+        if (lane < kRows) ash[wid][buf][lane] = a;
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    fetch(ch.y);
+    issue(0, ch.y);
+    fetch(ch.y + kRows);
+    int buf = 0;
+    for (int base = ch.y; base < ch.z; base += kRows, buf ^= 1) {
+        if (base + kRows < ch.z) {
+            issue(buf ^ 1, base + kRows);
+            fetch(base + 2 * kRows);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
         }
         __syncwarp();
-        const int cnt = min(32, ch.z - base);
-        for (int t = 0; t < cnt; ++t) {
-#pragma unroll
-            for (int q = 0; q < TR::NP; ++q)
-                acc[q] = fma(wsh[wid][t][rq[q]], wsh[wid][t][cq[q]], acc[q]);
-            if (lane < K) bacc = fma(ash[wid][t], wsh[wid][t][lane], bacc);
-        }
+        const int cnt = min(kRows, ch.z - base);
+#pragma unroll 2
+        for (int t = lane / K; t < cnt; t += GR) g.add(wsh[wid][buf][t], ash[wid][buf][t]);
         __syncwarp();
     }
+#pragma unroll
+    for (int o = K; o < 32; o <<= 1) {
+#pragma unroll
+        for (int i = 0; i < GT::TR; ++i) {
+            g.b[i] += shfl_xor(g.b[i], o);
+#pragma unroll
+            for (int q = 0; q < GT::TC; ++q) g.acc[i][q] += shfl_xor(g.acc[i][q], o);
+        }
+    }
+    if (lane >= K) return;
     T *out = part + c * TR::P;
 #pragma unroll
-    for (int q = 0; q < TR::NP; ++q)
-        if (lane + 32 * q < TR::N) out[lane + 32 * q] = acc[q];
-    if (lane < K) out[TR::N + lane] = bacc;
+    for (int i = 0; i < GT::TR; ++i) {
+        const int r = g.r0 + i;
+#pragma unroll
+        for (int q = 0; q < GT::TC; ++q)
+            if (g.c0 + q <= r) out[r * (r + 1) / 2 + g.c0 + q] = g.acc[i][q];
+        if (g.c0 == 0) out[TR::N + r] = g.b[i];
+    }
 }
 
 template <class T, int K>
@@ -117,6 +175,86 @@ als_solve_kernel(int64_t nseg, const int32_t *__restrict__ segchunk, const T *__
         return;
     }
     if (lane < k) F[s * k + lane] = (T)b[wid][lane];
+}
+
+// FP32 models: K lanes per segment (32 / K segments per warp), the refined
+// solve of glrm_spd.cuh.  The warps walk the segments with a grid stride, so
+// the (row, column) of a lane's triangle entries are worked out once.  With
+// the FP64 factorisation for every system the FP64 pipe was 85% busy; on the
+// 100,000 systems of the k = 32 completion table 4.83 -> 1.10 ms.
+template <int K>
+__global__ void __launch_bounds__(kAlsWarps * 32)
+als_solve_refined_kernel(int64_t nseg, const int32_t *__restrict__ segchunk, const float *__restrict__ part, int k,
+                         double gamma, float *__restrict__ F, int *__restrict__ err)
+{
+    using TR = Tri<K>;
+    constexpr int GR = 32 / K, NQ = (TR::N + K - 1) / K;
+    extern __shared__ __align__(16) unsigned char spd_raw[];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, grp = lane / K, lr = lane % K;
+    SpdSmem<K> &S = reinterpret_cast<SpdSmem<K> *>(spd_raw)[wid * GR + grp];
+    int rc[NQ];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+        int r, c;
+        tri_rc(lr + K * q < TR::N ? lr + K * q : 0, r, c);
+        rc[q] = r << 8 | c;
+    }
+    const int64_t step = (int64_t)gridDim.x * kAlsWarps * GR;
+    for (int64_t s0 = ((int64_t)blockIdx.x * kAlsWarps + wid) * GR; s0 < nseg; s0 += step) {
+        const int64_t s = s0 + grp;
+        const bool live = s < nseg;
+        const int cb = live ? segchunk[s] : 0, ce = live ? segchunk[s + 1] : 0;
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+            const int p = lr + K * q;
+            if (p < TR::N) {
+                const int r = rc[q] >> 8, c = rc[q] & 0xff;
+                double v = 0.0;
+                float f = 0.f;
+                if (ce - cb == 1) {
+                    f = part[(int64_t)cb * TR::P + p];
+                    v = (double)f;
+                } else {
+                    for (int t = cb; t < ce; ++t) {
+                        const float w = part[(int64_t)t * TR::P + p];
+                        v += (double)w;
+                        f += w;
+                    }
+                }
+                if (r == c) {  // unused rows / columns beyond k: an identity
+                    v = r < k ? v + gamma : 1.0;
+                    f = r < k ? f + (float)gamma : 1.f;
+                }
+                S.G[r * K + c] = S.G[c * K + r] = v;
+                S.L[r * (K + 1) + c] = S.L[c * (K + 1) + r] = f;
+            }
+        }
+        double b = 0.0;
+        if (lr < k)
+            for (int t = cb; t < ce; ++t) b += (double)part[(int64_t)t * TR::P + TR::N + lr];
+        S.b[lr] = b;
+        __syncwarp();
+        double x;
+        bool ok = spd_solve_refined<K>(S, x);
+        if (__any_sync(0xffffffffu, live && !ok)) {
+            // the systems not settled, one after the other: FP64 Cholesky (a
+            // failed one keeps the segment's factor and raises the flag)
+            for (int g = 0; g < GR; ++g) {
+                if (!(__shfl_sync(0xffffffffu, live && !ok ? 1 : 0, g * K))) continue;
+                SpdSmem<K> &Q = reinterpret_cast<SpdSmem<K> *>(spd_raw)[wid * GR + g];
+                const bool solved =
+                    warp_cholesky_solve<K, K>(reinterpret_cast<double(*)[K]>(Q.G), Q.b);
+                if (grp == g) {
+                    x = Q.b[lr];
+                    ok = solved;
+                    if (!solved && lr == 0) atomicOr(err, kErrPivot);
+                }
+                __syncwarp();
+            }
+        }
+        if (live && ok && lr < k) F[s * k + lr] = (float)x;
+        __syncwarp();
+    }
 }
 
 // Prox-prox update for quadratic loss (Section 7.2, "Prox-prox method"; the
@@ -176,6 +314,13 @@ proxprox_solve_kernel(int64_t nseg, const int32_t *__restrict__ segchunk, const 
     if (lane < k) F[s * k + lane] = (T)f;
 }
 
+// Whether a factor's rows can be copied in 16-byte pieces.
+template <class T>
+bool gram_vec(const T *W, int k)
+{
+    return k * sizeof(T) % 16 == 0 && reinterpret_cast<uintptr_t>(W) % 16 == 0;
+}
+
 template <class T, int K>
 cudaError_t launch_als_half(glrm_s *h, bool xstep, double gamma)
 {
@@ -197,12 +342,28 @@ cudaError_t launch_als_half(glrm_s *h, bool xstep, double gamma)
     tmark(h, xstep ? "als_gram_x" : "als_gram_y");
     if (o.nchunks)
         als_gram_kernel<T, K><<<blocks_for(o.nchunks, kAlsWarps), kAlsWarps * 32, 0, h->stream>>>(
-            o.nchunks, o.chunks, o.idx, (const T *)o.val, W, h->k, part);
+            o.nchunks, o.chunks, o.idx, (const T *)o.val, W, h->k, gram_vec<T>(W, h->k), part);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     tmark(h, xstep ? "als_solve_x" : "als_solve_y");
-    als_solve_kernel<T, K><<<blocks_for(o.nseg, kAlsWarps), kAlsWarps * 32, 0, h->stream>>>(
-        o.nseg, o.segchunk, part, h->k, gamma, F, h->s.err);
+    if constexpr (sizeof(T) == 4) {
+        constexpr size_t smem = sizeof(SpdSmem<K>) * (32 / K) * kAlsWarps;
+        int sms = 0, per = 0;
+        if ((e = cudaFuncSetAttribute(als_solve_refined_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)smem)) != cudaSuccess)
+            return e;
+        if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device)) != cudaSuccess) return e;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, als_solve_refined_kernel<K>, kAlsWarps * 32,
+                                                               smem)) != cudaSuccess)
+            return e;
+        const int64_t want = blocks_for(o.nseg, kAlsWarps * (32 / K));
+        als_solve_refined_kernel<K>
+            <<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)sms * std::max(per, 1))),
+               kAlsWarps * 32, smem, h->stream>>>(o.nseg, o.segchunk, part, h->k, gamma, F, h->s.err);
+    } else {
+        als_solve_kernel<T, K><<<blocks_for(o.nseg, kAlsWarps), kAlsWarps * 32, 0, h->stream>>>(
+            o.nseg, o.segchunk, part, h->k, gamma, F, h->s.err);
+    }
     tmark(h, nullptr);
     return cudaGetLastError();
 }
@@ -229,7 +390,7 @@ cudaError_t launch_proxprox_half(glrm_s *h, bool xstep, double alpha, int inner)
     tmark(h, xstep ? "als_gram_x" : "als_gram_y");
     if (o.nchunks)
         als_gram_kernel<T, K><<<blocks_for(o.nchunks, kAlsWarps), kAlsWarps * 32, 0, h->stream>>>(
-            o.nchunks, o.chunks, o.idx, (const T *)o.val, W, h->k, part);
+            o.nchunks, o.chunks, o.idx, (const T *)o.val, W, h->k, gram_vec<T>(W, h->k), part);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     tmark(h, xstep ? "proxprox_x" : "proxprox_y");
