@@ -151,8 +151,7 @@ __device__ bool spd_solve_refined(SpdSmem<K> &S, double &x)
         done = done || dm <= 0x1p-30f * xm;  // false for NaN
         if (__all_sync(0xffffffffu, done || !ok)) break;
     }
-    return __shfl_sync(0xffffffffu, ok && done ? 1 : 0, 0, K) != 0 &&
-           group_max<K>(ok ? 0.f : 1.f) == 0.f;
+    return ok && done;  // the same on every lane of the group: both follow from its shared values
 }
 
 }  // namespace glrm
