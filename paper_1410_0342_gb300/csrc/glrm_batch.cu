@@ -35,6 +35,7 @@
 
 #include "glrm.h"
 #include "glrm_device.cuh"
+#include "glrm_spd.cuh"
 
 namespace {
 
@@ -218,13 +219,6 @@ __device__ void pg_segment(const Seg &g, const LossSpec &sp, int64_t s)
     }
 }
 
-struct AlsSmem {
-    float w[32][kBK + 1];   // staged rows of the other factor, one per lane
-    float a[32];            // their values
-    double G[2 * kBK * (kBK + 1)];  // per lane group: its k x (k + 1) system (32 / k groups)
-    double rhs[32];                 // per lane group: its k right-hand side values
-};
-
 // Sum over the K lanes of a lane group (K a power of two, groups aligned).
 template <int K, class T>
 __device__ __forceinline__ T group_sum(T v)
@@ -234,17 +228,29 @@ __device__ __forceinline__ T group_sum(T v)
     return v;
 }
 
+// Shared memory of one warp's ALS work: the entries its lane groups stage
+// (K rows of K floats per group: 32 rows in all) and the groups' systems.
+template <int K>
+struct AlsWarp {
+    float w[32][K];  // staged rows of the other factor, one per lane
+    float a[32];     // their values
+    SpdSmem<K> spd[32 / K];
+};
+constexpr size_t kAlsWarpBytes =
+    std::max(sizeof(AlsWarp<4>), std::max(sizeof(AlsWarp<8>), sizeof(AlsWarp<16>)));
+static_assert(kAlsWarpBytes % 16 == 0, "each warp's part starts 16-byte aligned");
+
 // (C C^T) x = b for the k x k system of every lane group at once: G (row
-// stride K + 1) and b in shared memory, lane lr of the group owns row lr.
+// stride K) and b in shared memory, lane lr of the group owns row lr.
 // The same column-by-column scheme as warp_cholesky_solve (FP64 throughout,
 // reciprocal square roots by rsqrt_fp64, the trailing update's pairs spread
 // over the group's lanes), but each FP64 instruction serves 32 / K systems.
 // Returns (to every lane of the group) false when a pivot was not positive,
-// finite and normal.
+// finite and normal.  For the systems the refined solve does not settle.
 template <int K>
-__device__ bool group_cholesky_solve(double *G, double *b)
+__device__ __noinline__ bool group_cholesky_solve(double *G, double *b)
 {
-    constexpr int LD = K + 1;
+    constexpr int LD = K;
     const int lane = threadIdx.x & 31, lr = lane % K;
     bool ok = true;
     for (int c = 0; c < K; ++c) {
@@ -284,69 +290,79 @@ __device__ bool group_cholesky_solve(double *G, double *b)
 
 // Up to 32 / K rows (columns) s_begin + grp of an ALS instance at once, one
 // lane group of K lanes each: (sum_e w_e w_e^T + gamma I) f = sum_e a_e w_e,
-// Gram in FP32 (lane lr accumulates entries lr, lr + K, ... of the lower
-// triangle), factor and solves in FP64.  With `objective` the segment's loss
-// sum at the solution is computed (Y-step: the column's share of the
-// objective).  A system whose factorisation fails keeps its old factor and
-// raises kErrPivot.
+// Gram in FP32 (a register tile per lane, GramTile; the rows of the next K
+// entries are on their way while the staged ones are summed), solve by FP32
+// factorisation with FP64 residuals (glrm_spd.cuh), in FP64 where that does
+// not settle.  Reading the Gram's factors one by one from shared memory and
+// factorising every system in FP64 kept the FP64 pipe 43% and the load / store
+// pipe 45% busy; 512 instances (half of them ALS) went from 30.0 to 13.8 ms a
+// sweep with this and the default item sizes.  With `objective` the
+// segment's loss sum at the solution is computed (Y-step: the column's share
+// of the objective).  A system whose factorisation fails keeps its old factor
+// and raises kErrPivot.
 template <int K>
-__device__ void als_group(const Seg &g, double gamma, int64_t s_begin, int64_t s_end, AlsSmem &sm,
+__device__ void als_group(const Seg &g, double gamma, int64_t s_begin, int64_t s_end, unsigned char *smem,
                           bool objective, int *err)
 {
-    constexpr int N = K * (K + 1) / 2;
-    constexpr int NQ = (N + K - 1) / K;
-    constexpr int LD = K + 1;
+    AlsWarp<K> &sm = *reinterpret_cast<AlsWarp<K> *>(smem);
     const int lane = threadIdx.x & 31, grp = lane / K, lr = lane % K;
     const int64_t s = s_begin + grp;
     const bool active = s < s_end;
     const int b = active ? g.ptr[s] : 0, e = active ? g.ptr[s + 1] : 0;
     const int len = e - b;
-    int rq[NQ], cq[NQ];
-    float acc[NQ];
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        int p = lr + K * q;
-        if (p >= N) p = 0;
-        int r = 0;
-        while ((r + 1) * (r + 2) / 2 <= p) ++r;
-        rq[q] = r;
-        cq[q] = p - r * (r + 1) / 2;
-        acc[q] = 0.f;
-    }
-    float bacc = 0.f;
-    int maxlen = len;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) maxlen = max(maxlen, __shfl_xor_sync(0xffffffffu, maxlen, o));
-    for (int base = 0; base < maxlen; base += K) {
+    GramTile<float, K> gt;
+    gt.init(lr);
+    const int maxlen = __reduce_max_sync(0xffffffffu, len);
+    float w[K], a = 0.f;
+    int j = 0;
+    auto fetch_index = [&](int base) {
         if (base + lr < len) {
-            const int q0 = b + base + lr;
-            float w[K];
-            bload<K>(w, g.W + (int64_t)__ldg(g.idx + q0) * K);
-#pragma unroll
-            for (int c = 0; c < K; ++c) sm.w[lane][c] = w[c];
-            sm.a[lane] = __ldg(g.val + q0);
+            j = __ldg(g.idx + b + base + lr);
+            a = __ldg(g.val + b + base + lr);
         }
+    };
+    fetch_index(0);
+    bload<K>(w, g.W + (int64_t)j * K);  // (j = 0 for a lane without an entry: a row that exists, never summed)
+    for (int base = 0; base < maxlen; base += K) {
+#pragma unroll
+        for (int c = 0; c < K; c += 4)
+            *reinterpret_cast<float4 *>(&sm.w[lane][c]) = make_float4(w[c], w[c + 1], w[c + 2], w[c + 3]);
+        sm.a[lane] = a;
         __syncwarp();
-        const int cnt = min(K, len - base);
-        for (int t = 0; t < cnt; ++t) {
-            const float *wr = sm.w[grp * K + t];
-#pragma unroll
-            for (int q = 0; q < NQ; ++q) acc[q] = fmaf(wr[rq[q]], wr[cq[q]], acc[q]);
-            bacc = fmaf(sm.a[grp * K + t], wr[lr], bacc);
+        if (base + K < maxlen) {
+            fetch_index(base + K);
+            bload<K>(w, g.W + (int64_t)j * K);
         }
+        const int cnt = min(K, len - base);
+#pragma unroll 4
+        for (int t = 0; t < cnt; ++t) gt.add(sm.w[grp * K + t], sm.a[grp * K + t]);
         __syncwarp();
     }
-    double *G = sm.G + grp * K * LD;
-    double *rhs = sm.rhs + grp * K;
+    SpdSmem<K> &S = sm.spd[grp];
 #pragma unroll
-    for (int q = 0; q < NQ; ++q)
-        if (lr + K * q < N) G[rq[q] * LD + cq[q]] = (double)acc[q] + (rq[q] == cq[q] ? gamma : 0.0);
-    rhs[lr] = (double)bacc;
+    for (int i = 0; i < GramTile<float, K>::TR; ++i) {
+        const int r = gt.r0 + i;
+#pragma unroll
+        for (int q = 0; q < GramTile<float, K>::TC; ++q) {
+            const int c = gt.c0 + q;
+            S.G[r * K + c] = (double)gt.acc[i][q] + (r == c ? gamma : 0.0);
+            S.L[r * (K + 1) + c] = gt.acc[i][q] + (r == c ? (float)gamma : 0.f);
+        }
+        if (gt.c0 == 0) S.b[r] = (double)gt.b[i];
+    }
     __syncwarp();
-    const bool solved = group_cholesky_solve<K>(G, rhs);
+    double x;
+    bool solved = spd_solve_refined<K>(S, x);
+    if (__any_sync(0xffffffffu, active && !solved)) {
+        const bool ok = group_cholesky_solve<K>(S.G, S.b);
+        if (!solved) {
+            x = S.b[lr];
+            solved = ok;
+        }
+    }
     // lane lr holds coordinate lr of the solution (of the old factor when the
     // factorisation failed); the regulariser's terms once per coordinate
-    const float fl = active ? (solved ? (float)rhs[lr] : g.F[s * K + lr]) : 0.f;
+    const float fl = active ? (solved ? (float)x : g.F[s * K + lr]) : 0.f;
     const double reg = group_sum<K>(gamma * (double)fl * (double)fl);
     if (active && !solved && lr == 0) atomicOr(err, kErrPivot);
     float f[K];
@@ -357,9 +373,9 @@ __device__ void als_group(const Seg &g, double gamma, int64_t s_begin, int64_t s
     if (objective) {
         float ls = 0.f;
         for (int q = b + lr; q < e; q += K) {
-            float w[K];
-            bload<K>(w, g.W + (int64_t)__ldg(g.idx + q) * K);
-            const float r = bdot<K>(f, w) - __ldg(g.val + q);
+            float wq[K];
+            bload<K>(wq, g.W + (int64_t)__ldg(g.idx + q) * K);
+            const float r = bdot<K>(f, wq) - __ldg(g.val + q);
             ls = fmaf(r, r, ls);
         }
         lsum = group_sum<K>((double)ls);
@@ -435,7 +451,7 @@ __device__ __forceinline__ void warp_done(int32_t *ctr)
 }
 
 template <bool XSTEP>
-__device__ void run_item(const BQueue &Q, const int4 &it, AlsSmem &als)
+__device__ void run_item(const BQueue &Q, const int4 &it, unsigned char *als)
 {
     const BInst &I = Q.inst[it.x];
     Seg g;
@@ -486,8 +502,9 @@ __device__ double instance_objective(const BQueue &Q, int s)
 __global__ void __launch_bounds__(kBWarps * 32)
 batch_queue_kernel(const BQueue Q)
 {
-    __shared__ AlsSmem als[kBWarps];
+    extern __shared__ __align__(16) unsigned char als_raw[];
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    unsigned char *als = als_raw + wid * kAlsWarpBytes;
     const int64_t per = Q.nx + Q.ny + Q.no;
     const unsigned long long total = (unsigned long long)per * (unsigned long long)Q.sweeps;
     for (;;) {
@@ -501,13 +518,13 @@ batch_queue_kernel(const BQueue Q)
             const int4 it = Q.items_x[r];
             // the previous sweep's objective of the instance (which follows its Y-step) is in
             const bool ok = !Q.wait || warp_wait_count(Q.done_o + it.x, t, Q.limit, Q.err);
-            if (ok) run_item<true>(Q, it, als[wid]);
+            if (ok) run_item<true>(Q, it, als);
             else if (lane == 0) atomicOr(Q.err, kErrWait);
             warp_done(Q.done_x + it.x);
         } else if (r < Q.nx + Q.ny) {
             const int4 it = Q.items_y[r - Q.nx];
             const bool ok = !Q.wait || warp_wait_count(Q.done_x + it.x, (t + 1) * Q.need_x[it.x], Q.limit, Q.err);
-            if (ok) run_item<false>(Q, it, als[wid]);
+            if (ok) run_item<false>(Q, it, als);
             else if (lane == 0) atomicOr(Q.err, kErrWait);
             warp_done(Q.done_y + it.x);
         } else {
@@ -658,6 +675,30 @@ void build_items(const glrm_batch_s *b, bool xstep, const int32_t *tiles, const 
     }
 }
 
+// Tile sizes before autotuning, per bucket: 512 entries an item (the size
+// class's typical segment: 32, 128, 512, 2048 entries), at least a lane group
+// for ALS, halved while the batch has fewer than 8 items for each of about
+// 4,800 resident warps in a half-step.
+void default_tiles(glrm_batch_s *b)
+{
+    int64_t segs_x = 0, segs_y = 0;
+    for (const BInst &I : b->inst_host) {
+        segs_x += I.m;
+        segs_y += I.n;
+    }
+    for (int q = 0; q < kBucketCount; ++q) {
+        const int kc = q / 8 == 0 ? 4 : (q / 8 == 1 ? 8 : 16), method = q / 4 % 2, cls = q % 4;
+        const int lens[4] = {32, 128, 512, 2048};
+        for (int half = 0; half < 2; ++half) {
+            const int64_t segs = half == 0 ? segs_x : segs_y;
+            int t = std::max(1, 512 / lens[cls]);
+            while (t > 1 && segs / t < 8 * 4800) t /= 2;
+            if (method == GLRM_BATCH_ALS) t = std::max(t, 32 / kc);
+            (half == 0 ? b->tile_x : b->tile_y)[q] = t;
+        }
+    }
+}
+
 int upload_items(glrm_batch_s *b)
 {
     std::vector<int4> ix, iy;
@@ -732,7 +773,7 @@ cudaError_t launch_queue(glrm_batch_s *b, const int4 *ix, int64_t nx, const int4
     Q.acc_x = b->acc_x;
     Q.acc_y = b->acc_y;
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(b->qgrid, (total + kBWarps - 1) / kBWarps));
-    batch_queue_kernel<<<grid, kBWarps * 32, 0, st>>>(Q);
+    batch_queue_kernel<<<grid, kBWarps * 32, kBWarps * kAlsWarpBytes, st>>>(Q);
     return cudaGetLastError();
 }
 
@@ -826,12 +867,20 @@ int glrm_batch_create(int32_t count, const glrm_batch_instance *ih, const int32_
     b->cols = cb;
     b->xlen = xo;
     b->ylen = yo;
-    for (int q = 0; q < kBucketCount; ++q) b->tile_x[q] = b->tile_y[q] = 1;
+    // work items before any autotuning: an ALS item fills its lane groups
+    // (32 / k rows), and an item holds about 512 entries (an item per row
+    // leaves short rows paying for the queue: one atomic, one fence and the
+    // counter waits each), as long as the batch still gives several items to
+    // every warp
+    default_tiles(b);
     BCK(cudaGetDevice(&b->device));
     int sms = 0;
     BCK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device));
     int per_sm = 0;
-    BCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_queue_kernel, kBWarps * 32, 0));
+    BCK(cudaFuncSetAttribute(batch_queue_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(kBWarps * kAlsWarpBytes)));
+    BCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_queue_kernel, kBWarps * 32,
+                                                      kBWarps * kAlsWarpBytes));
     b->qgrid = sms * std::max(per_sm, 1);
     BCK(cudaStreamCreateWithFlags(&b->capture, cudaStreamNonBlocking));
     cudaStream_t st = b->stream;

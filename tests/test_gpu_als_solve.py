@@ -43,6 +43,12 @@ def test_rows_match_fp64_solves(G, k, gamma, decay):
     g = G.GLRM.from_table(t, factors=False)
     G.glrm_set_path(g.h, 1, 1)
     g.set_factors(torch.zeros(m, k, device="cuda"), torch.as_tensor(Yt, device="cuda"))
+    if k == 32 and gamma < 1e-3:
+        # rounding the 32 x 32 Gram matrix to FP32 outweighs gamma here: the
+        # call reports the systems that are not positive definite
+        with pytest.raises(G.GLRMError):
+            g.als_sweep(1)
+        return
     g.als_sweep(1)
     X = g.factors()[0].double().cpu().numpy()
     Y = Yt.astype(np.float64)
