@@ -485,7 +485,9 @@ int glrm_set_state(glrm_t h, const void *buf_host, size_t len);
 
 /* Kernel path of each half-step (a tuning knob; results agree to rounding).
  *   GLRM_PATH_CHUNKED  entries cut into chunks of <= 1024, one warp each; the
- *                      other factor read from global memory (any k, any size)
+ *                      other factor read from global memory (any k, any size);
+ *                      one launch per half-step when no segment is longer
+ *                      than a chunk
  *   GLRM_PATH_FUSED    the whole other factor staged in each CTA's shared
  *                      memory by a TMA bulk copy; one warp runs a row's (column's)
  *                      gradient, prox, re-evaluation and decision in one kernel
@@ -509,7 +511,7 @@ int glrm_set_state(glrm_t h, const void *buf_host, size_t len);
  * GLRM_PATH_AUTO picks dense for FP32 and BF16 models with k <= 64 when at least 40% of
  * the cells are observed (and the dense copy takes at most half the free
  * device memory); otherwise masked when a tile's pairs average >= 8 observed
- * lanes, else fused when the other factor fits, else blocked when a
+ * lanes (chunked when that gives fewer than 48 units of work), else fused when the other factor fits, else blocked when a
  * (panel, segment) run holds >= 64 entries on average, else chunked.  The
  * staged paths need k <= 32.  glrm_set_path(h, xstep_path, ystep_path) may be
  * called before or after glrm_set_observed; an infeasible request returns

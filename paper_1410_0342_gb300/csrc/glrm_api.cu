@@ -71,7 +71,7 @@ void free_scratch(Scratch &s, cudaStream_t st)
     dfree(s.part_grad, st); dfree(s.part_loss, st); dfree(s.part_loss2, st); dfree(s.cand, st);
     dfree(s.f_old, st); dfree(s.r_old, st); dfree(s.r_new, st);
     dfree(s.kept_obj_x, st); dfree(s.kept_reg_x, st); dfree(s.kept_obj_y, st); dfree(s.kept_reg_y, st);
-    dfree(s.acc_x, st); dfree(s.acc_y, st); dfree(s.red_part, st); dfree(s.red_cnt, st);
+    dfree(s.acc_x, st); dfree(s.acc_y, st); dfree(s.red_part, st); dfree(s.red_cnt, st); dfree(s.ticket, st);
     dfree(s.hist, st); dfree(s.accepts, st); dfree(s.scalar, st); dfree(s.als_part, st); dfree(s.err, st);
     dfree(s.x_bf16, st); dfree(s.yt_bf16, st);
     dfree(s.conv, st); dfree(s.conv_par, st); dfree(s.conv_cnt, st);
@@ -125,12 +125,17 @@ int tiled_width(int k)
 // other factor (plus, for the X-step, its loss table) fits in one CTA's shared
 // memory; blocked when panels of it do and a (panel, segment) run holds 64
 // entries or more on average; chunked otherwise.
+// Units (warps) below which the automatic choice prefers the chunked form to
+// masked tiles: on the 200 x 100, k = 5 FP64 table (7 and 4 units) the masked
+// half-steps take 200 and 272 us, the chunked ones 18 and 23 us.
+constexpr int64_t kMaskedMinUnits = 48;
+
 // Masked tiles: count each tile's pairs; build the layout when forced or when
 // a pair averages >= 8 observed lanes.  The other factor is kept whole in
 // shared memory when it fits, else gathered per batch (needs k == K).  Tiles
 // are split into units of P pairs only when there are too few tiles to give
 // every warp of the GPU one.
-int plan_masked(glrm_s *h, Orient &o, bool xstep, int force, int K, int sms, size_t budget)
+int plan_masked(glrm_s *h, Orient &o, bool xstep, int force, int K, int sms, size_t budget, bool &small)
 {
     const size_t es = elem_size(h->prec);
     const int64_t nother = xstep ? h->n : h->m;
@@ -190,6 +195,16 @@ int plan_masked(glrm_s *h, Orient &o, bool xstep, int force, int K, int sms, siz
         nunits += nu;
     }
     ubeg[ntiles] = (int32_t)nunits;
+    // A warp per tile leaves a small orientation on a few warps, each walking
+    // its whole pair list: below kMaskedMinUnits the chunked form (a warp per
+    // segment, 32 times the warps) is taken.
+    if (!forced && nunits < kMaskedMinUnits) {
+        small = true;
+        return give_up("");
+    }
+    // fewer units than the GPU has warps: one or a few warps per CTA, so that
+    // the units spread over the SMs
+    warps = (int)std::min<int64_t>(warps, std::max<int64_t>(1, (nunits + sms - 1) / sms));
     o.full = full;
     o.warps = warps;
     o.P = (int)P;
@@ -257,8 +272,9 @@ int choose_mode(glrm_s *h, Orient &o, bool xstep, int force)
     const size_t per_row = (size_t)K * es + (xstep ? sizeof(LossSpec) : 0);
     const size_t budget = (size_t)optin - 1024;
     if (force == GLRM_PATH_AUTO || force == GLRM_PATH_MASKED || force == GLRM_PATH_MASKED_SPLIT) {
-        int rc = plan_masked(h, o, xstep, force, K, sms, budget);
-        if (rc != GLRM_OK || o.mode == kModeMasked || force != GLRM_PATH_AUTO) return rc;
+        bool small = false;  // dense enough for masked tiles, but too few of them
+        int rc = plan_masked(h, o, xstep, force, K, sms, budget, small);
+        if (rc != GLRM_OK || o.mode == kModeMasked || force != GLRM_PATH_AUTO || small) return rc;
     }
     // per warp: two staging buffers of `cap` (index, value) pairs
     const size_t per_cap = (size_t)kStreamWarps * 2 * (sizeof(int32_t) + es);
@@ -396,6 +412,8 @@ int alloc_scratch(glrm_s *h)
     CK(dalloc(h, &s.acc_y, (size_t)h->n * sizeof(int32_t)));
     CK(dalloc(h, &s.red_part, kRedBlocks * sizeof(double)));
     CK(dalloc(h, &s.red_cnt, 2 * kRedBlocks * sizeof(long long)));
+    CK(dalloc(h, &s.ticket, sizeof(unsigned)));
+    CK(cudaMemsetAsync(s.ticket, 0, sizeof(unsigned), h->stream));
     CK(dalloc(h, &s.accepts, 2 * sizeof(long long)));
     CK(dalloc(h, &s.scalar, sizeof(double)));
     CK(dalloc(h, &s.err, sizeof(int)));

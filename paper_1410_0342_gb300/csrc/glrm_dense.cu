@@ -1558,15 +1558,13 @@ cudaError_t dense_objective_at(glrm_s *h, const float *X, const float *Yt, doubl
     if (e != cudaSuccess) return e;
     tmark(h, "dense_objective");
     if ((e = launch_dense<true, false>(h, X, nullptr, s.part_loss)) != cudaSuccess) return e;
-    tmark(h, "reduce_stage1");
-    reduce_stage1<float><<<kRedBlocks, 256, 0, h->stream>>>(
+    tmark(h, "reduce");
+    reduce_kernel<float><<<reduce_blocks(h->dn.slots_x + (h->m + h->n) * h->k), 256, 0, h->stream>>>(
         s.part_loss, h->dn.slots_x, nullptr, 0, X, h->m, reg_code(h, true), (float)h->rx_w, Yt, h->n,
-        reg_code(h, false), (float)h->ry_w, h->k, nullptr, 0, nullptr, 0, s.red_part, s.red_cnt);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    tmark(h, "reduce_stage2");
-    reduce_stage2<<<1, 256, 0, h->stream>>>(s.red_part, s.red_cnt, kRedBlocks, out, nullptr);
+        reg_code(h, false), (float)h->ry_w, h->k, nullptr, 0, nullptr, 0, s.red_part, s.red_cnt, s.ticket, out,
+        nullptr);
     tmark(h, nullptr);
-    h->launches += 2;
+    h->launches += 1;
     return cudaGetLastError();
 }
 

@@ -14,6 +14,8 @@
 //   decide_kernel        per segment: keep f+ (alpha *= 1.05) if
 //                        f_new <= f_old, else keep f (alpha *= 0.7)
 // Chunks hold at most kChunk entries, so long columns spread over many warps.
+// Where no segment of an orientation is longer than one chunk, seg_kernel runs
+// all four steps of a segment in one warp and one launch.
 // All reductions run in a fixed order: results are bitwise reproducible.
 #pragma once
 
@@ -252,6 +254,160 @@ pass_kernel(int64_t nchunks, const int4 *__restrict__ chunks, const int32_t *__r
     if (lane == 0) part_loss[c] = ls;
 }
 
+// A whole half-step of segments that fit in one chunk, a warp per segment:
+// gradient pass, prox, loss pass of the candidate, decision.  The candidate's
+// coordinates stay in the lanes that hold the gradient's (every lane group
+// has the whole row), so nothing goes through memory between the steps: one
+// launch of the four and no partials.  On the 200 x 100, k = 5 FP64 table,
+// whose half-steps are launch- and latency-bound, 18 and 23 us (masked tiles:
+// 200 and 272 us); 10.6 -> 10.3 ms for the 1,000,000 rows (200 entries, k = 64)
+// of the completion table.
+template <class T, int K, bool XSTEP, bool VEC>
+__global__ void __launch_bounds__(kWarpsPerBlock * 32)
+seg_kernel(int64_t nseg, const int32_t *__restrict__ ptr, const int32_t *__restrict__ idx,
+           const T *__restrict__ val, T *__restrict__ F, const T *__restrict__ W, int k,
+           const LossOf<T> *__restrict__ loss, T *__restrict__ alpha, int rkind, T rw,
+           double *__restrict__ kept_obj, double *__restrict__ kept_reg, int32_t *__restrict__ accepted,
+           const T *__restrict__ lsc)
+{
+    using LN = Lanes<K>;
+    constexpr int G = LN::G, S = LN::S, PER = LN::PER;
+    constexpr int VW = unit_of<T>();
+    const int lane = threadIdx.x & 31;
+    const int64_t s = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (s >= nseg) return;  // the whole warp leaves together
+    const int gl = lane % G, grp = lane / G;
+    const int b = ptr[s], e = ptr[s + 1];
+    const T al = alpha[s];
+    T f[S], g[S];
+    load_lane<T, S, G, VW, VEC>(f, F + s * k, gl, k);
+#pragma unroll
+    for (int q = 0; q < S; ++q) g[q] = T(0);
+    LossOf<T> sp;
+    T wsc = T(1);
+    if constexpr (!XSTEP) {
+        sp = loss[s];
+        if (lsc) wsc = __ldg(lsc + s);
+    }
+    // loss (and derivative) of entry q at f, its row in w
+    auto entry = [&](int q, const T (&x)[S], T (&w)[S], T &L) -> T {
+        const bool in = q < e;
+        int j = 0;
+        T a = T(0);
+        if (in) {
+            j = __ldg(idx + q);
+            a = __ldg(val + q);
+            load_lane<T, S, G, VW, VEC>(w, W + (int64_t)j * k, gl, k);
+        } else {
+#pragma unroll
+            for (int c = 0; c < S; ++c) w[c] = T(0);
+        }
+        T u = T(0);
+#pragma unroll
+        for (int c = 0; c < S; ++c) u = fma(x[c], w[c], u);
+#pragma unroll
+        for (int o = 1; o < G; o <<= 1) u += shfl_xor(u, o);
+        T d = T(0);
+        L = T(0);
+        if (in) {
+            if constexpr (XSTEP) {
+                sp = loss[j];
+                if (lsc) wsc = __ldg(lsc + j);
+            }
+            d = loss_deriv<T>(sp, u, a, L);
+            if (lsc) {
+                d *= wsc;
+                L *= wsc;
+            }
+        }
+        return d;
+    };
+    T lsum = T(0);
+    for (int q = b; q < e; q += PER) {
+        T w[S], L;
+        const T d = entry(q + grp, f, w, L);
+#pragma unroll
+        for (int c = 0; c < S; ++c) g[c] = fma(d, w[c], g[c]);
+        if (gl == 0) lsum += L;
+    }
+#pragma unroll
+    for (int c = 0; c < S; ++c) {
+#pragma unroll
+        for (int o = G; o < 32; o <<= 1) g[c] += shfl_xor(g[c], o);
+    }
+    const double fo_loss = warp_sum((double)lsum);
+    // the candidate, in the lanes' own coordinates
+    T ro = T(0), rn = T(0);
+#pragma unroll
+    for (int c = 0; c < S; ++c) {
+        const int cc = slot_coord<S, G, VW, VEC>(c, gl);
+        if (cc < k) {
+            const int rkc = reg_kind_at(rkind, cc, k);
+            const T xp = prox1<T>(rkc, rw, al, f[c] - al * g[c]);
+            ro += reg1t<T>(rkc, rw, f[c]);
+            rn += reg1t<T>(rkc, rw, xp);
+            f[c] = xp;
+        }
+    }
+#pragma unroll
+    for (int o = 1; o < G; o <<= 1) {
+        ro += shfl_xor(ro, o);
+        rn += shfl_xor(rn, o);
+    }
+    // losses of the candidate, the next group of entries on its way while the
+    // current one is evaluated (as in the loss passes of pass_kernel)
+    T lsum2 = T(0);
+    T an = T(0), wn[S], wscn = wsc;
+    LossOf<T> spn = sp;
+    auto fetch = [&](int q) {
+        if (q < e) {
+            const int j = __ldg(idx + q);
+            an = __ldg(val + q);
+            load_lane<T, S, G, VW, VEC>(wn, W + (int64_t)j * k, gl, k);
+            if constexpr (XSTEP) {
+                spn = loss[j];
+                if (lsc) wscn = __ldg(lsc + j);
+            }
+        } else {
+#pragma unroll
+            for (int c = 0; c < S; ++c) wn[c] = T(0);
+        }
+    };
+    fetch(b + grp);
+    for (int q = b; q < e; q += PER) {
+        const T a = an;
+        T u = T(0);
+#pragma unroll
+        for (int c = 0; c < S; ++c) u = fma(f[c], wn[c], u);
+        sp = spn;
+        wsc = wscn;
+        fetch(q + PER + grp);
+#pragma unroll
+        for (int o = 1; o < G; o <<= 1) u += shfl_xor(u, o);
+        if (q + grp < e) {
+            T L;
+            loss_deriv<T>(sp, u, a, L);
+            if (lsc) L *= wsc;
+            if (gl == 0) lsum2 += L;
+        }
+    }
+    const double fn = warp_sum((double)lsum2) + rn, fo = fo_loss + ro;
+    const bool acc = fn <= fo;
+    if (acc && grp == 0) {
+#pragma unroll
+        for (int c = 0; c < S; ++c) {
+            const int cc = slot_coord<S, G, VW, VEC>(c, gl);
+            if (cc < k) F[s * k + cc] = f[c];
+        }
+    }
+    if (lane == 0) {
+        alpha[s] = al * (acc ? T(1.05) : T(0.7));
+        kept_obj[s] = acc ? fn : fo;
+        kept_reg[s] = acc ? rn : ro;
+        accepted[s] = acc ? 1 : 0;
+    }
+}
+
 // Round FP32 values to BF16 (round to nearest even).
 static __global__ void to_bf16_kernel(const float *__restrict__ src, int64_t n, __nv_bfloat16 *__restrict__ dst)
 {
@@ -465,24 +621,43 @@ cudaError_t launch_decide(int64_t nseg, const int32_t *segchunk, const double *p
     return cudaGetLastError();
 }
 
-// Deterministic two-level sums.  Stage 1: block b sums a fixed contiguous
-// range of each source; stage 2: one block sums the kRedBlocks partials.
+// Deterministic two-level sums in one launch: block b sums a fixed contiguous
+// range of each source; the block that finishes last (a counter, reset for the
+// next launch) sums the blocks' partials in block order.  (As two launches the
+// second took 6 us to sum 304 values.)
 template <class T>
 __global__ void __launch_bounds__(256)
-reduce_stage1(const double *__restrict__ a, int64_t na, const double *__restrict__ b, int64_t nb,
+reduce_kernel(const double *__restrict__ a, int64_t na, const double *__restrict__ b, int64_t nb,
               const T *__restrict__ X, int64_t m, int rxk, T rxw, const T *__restrict__ Yt,
               int64_t n, int ryk, T ryw, int k, const int32_t *__restrict__ ca, int64_t nca,
               const int32_t *__restrict__ cb, int64_t ncb, double *__restrict__ part,
-              long long *__restrict__ cnt)
+              long long *__restrict__ cnt, unsigned *__restrict__ ticket, double *__restrict__ out,
+              long long *__restrict__ cnt_out)
 {
     __shared__ double sh[256];
     __shared__ long long shc[2][256];
+    __shared__ bool last;
     double v = 0.0;
     long long c1 = 0, c2 = 0;
     auto range = [&](int64_t len, int64_t &lo, int64_t &hi) {
         const int64_t per = (len + gridDim.x - 1) / gridDim.x;
         lo = per * blockIdx.x;
         hi = lo + per < len ? lo + per : len;
+    };
+    auto block_sums = [&]() {  // sums of v, c1, c2 over the block, on thread 0
+        __syncthreads();
+        sh[threadIdx.x] = v;
+        shc[0][threadIdx.x] = c1;
+        shc[1][threadIdx.x] = c2;
+        __syncthreads();
+        for (int o = 128; o > 0; o >>= 1) {
+            if (threadIdx.x < o) {
+                sh[threadIdx.x] += sh[threadIdx.x + o];
+                shc[0][threadIdx.x] += shc[0][threadIdx.x + o];
+                shc[1][threadIdx.x] += shc[1][threadIdx.x + o];
+            }
+            __syncthreads();
+        }
     };
     int64_t lo, hi;
     if (a) { range(na, lo, hi); for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) v += a[i]; }
@@ -499,57 +674,40 @@ reduce_stage1(const double *__restrict__ a, int64_t na, const double *__restrict
     }
     if (ca) { range(nca, lo, hi); for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) c1 += ca[i]; }
     if (cb) { range(ncb, lo, hi); for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) c2 += cb[i]; }
-    sh[threadIdx.x] = v;
-    shc[0][threadIdx.x] = c1;
-    shc[1][threadIdx.x] = c2;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o) {
-            sh[threadIdx.x] += sh[threadIdx.x + o];
-            shc[0][threadIdx.x] += shc[0][threadIdx.x + o];
-            shc[1][threadIdx.x] += shc[1][threadIdx.x + o];
-        }
-        __syncthreads();
-    }
+    block_sums();
     if (threadIdx.x == 0) {
         part[blockIdx.x] = sh[0];
         cnt[2 * blockIdx.x] = shc[0][0];
         cnt[2 * blockIdx.x + 1] = shc[1][0];
+        __threadfence();
+        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
     }
-}
-
-static __global__ void __launch_bounds__(256)
-reduce_stage2(const double *__restrict__ part, const long long *__restrict__ cnt, int nparts,
-              double *__restrict__ out, long long *__restrict__ cnt_out)
-{
-    __shared__ double sh[256];
-    __shared__ long long shc[2][256];
-    double v = 0.0;
-    long long c1 = 0, c2 = 0;
-    for (int i = threadIdx.x; i < nparts; i += blockDim.x) {
-        v += part[i];
-        c1 += cnt[2 * i];
-        c2 += cnt[2 * i + 1];
-    }
-    sh[threadIdx.x] = v;
-    shc[0][threadIdx.x] = c1;
-    shc[1][threadIdx.x] = c2;
     __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o) {
-            sh[threadIdx.x] += sh[threadIdx.x + o];
-            shc[0][threadIdx.x] += shc[0][threadIdx.x + o];
-            shc[1][threadIdx.x] += shc[1][threadIdx.x + o];
-        }
-        __syncthreads();
+    if (!last) return;
+    __threadfence();
+    v = 0.0;
+    c1 = c2 = 0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) {
+        v += __ldcg(part + i);
+        c1 += __ldcg(cnt + 2 * i);
+        c2 += __ldcg(cnt + 2 * i + 1);
     }
+    block_sums();
     if (threadIdx.x == 0) {
         if (out) *out = sh[0];
         if (cnt_out) {
             cnt_out[0] = shc[0][0];
             cnt_out[1] = shc[1][0];
         }
+        *ticket = 0u;
     }
+}
+
+// Blocks of a reduction over `items` values: one per 1,024 values, at most
+// kRedBlocks (a small table's sum is not spread over 304 blocks).
+inline unsigned reduce_blocks(int64_t items)
+{
+    return (unsigned)std::max<int64_t>(1, std::min<int64_t>(kRedBlocks, (items + 1023) / 1024));
 }
 
 // Gradient of each segment: sum of its chunk partials (+ the regulariser's
@@ -653,6 +811,46 @@ cudaError_t dispatch_pass(const Orient &o, const T *F, const WT *W, int k, const
     return cudaErrorInvalidValue;
 }
 
+template <class T, int K, bool XSTEP>
+cudaError_t launch_seg(glrm_s *h, const Orient &o, T *F, const T *W, T *alpha, int rk, T rw)
+{
+    Scratch &s = h->s;
+    const bool vec = h->k == K && (reinterpret_cast<uintptr_t>(F) | reinterpret_cast<uintptr_t>(W)) % 16 == 0;
+    // few segments: fewer warps per block, so that they spread over the SMs
+    int warps = kWarpsPerBlock;
+    while (warps > 1 && o.nseg < 152LL * warps) warps /= 2;
+    const unsigned nb = blocks_for(o.nseg, warps);
+    auto go = [&](auto kern) {
+        kern<<<nb, warps * 32, 0, h->stream>>>(
+            o.nseg, o.ptr, o.idx, (const T *)o.val, F, W, h->k, loss_of<T>(h), alpha, rk, rw,
+            XSTEP ? s.kept_obj_x : s.kept_obj_y, XSTEP ? s.kept_reg_x : s.kept_reg_y, XSTEP ? s.acc_x : s.acc_y,
+            (const T *)h->lscale);
+    };
+    if (vec) go(seg_kernel<T, K, XSTEP, true>);
+    else go(seg_kernel<T, K, XSTEP, false>);
+    h->launches += 1;
+    return cudaGetLastError();
+}
+
+template <class T, bool XSTEP>
+cudaError_t dispatch_seg(glrm_s *h, const Orient &o, T *F, const T *W, T *alpha, int rk, T rw)
+{
+    const int k = h->k;
+#define GLRM_SEG_CASE(KK) \
+    if (k <= KK) return launch_seg<T, KK, XSTEP>(h, o, F, W, alpha, rk, rw);
+    GLRM_SEG_CASE(4)
+    GLRM_SEG_CASE(8)
+    GLRM_SEG_CASE(12)
+    GLRM_SEG_CASE(16)
+    GLRM_SEG_CASE(20)
+    GLRM_SEG_CASE(24)
+    GLRM_SEG_CASE(32)
+    GLRM_SEG_CASE(48)
+    GLRM_SEG_CASE(64)
+#undef GLRM_SEG_CASE
+    return cudaErrorInvalidValue;
+}
+
 template <class T>
 cudaError_t Engine<T>::half_step(glrm_s *h, bool xstep)
 {
@@ -669,6 +867,12 @@ cudaError_t Engine<T>::half_step(glrm_s *h, bool xstep)
     cudaError_t e;
     if constexpr (std::is_same<T, float>::value) {
         if (h->prec == GLRM_BF16) return bf16_half_step_entry(h, xstep);
+    }
+    if (o.maxlen <= kChunk) {
+        tmark(h, xstep ? "seg_x" : "seg_y");
+        e = xstep ? dispatch_seg<T, true>(h, o, F, W, alpha, rk, rw) : dispatch_seg<T, false>(h, o, F, W, alpha, rk, rw);
+        tmark(h, nullptr);
+        return e;
     }
     tmark(h, xstep ? "pass_grad_x" : "pass_grad_y");
     const T *lsc = (const T *)h->lscale;
@@ -700,16 +904,12 @@ template <class T>
 cudaError_t Engine<T>::reduce_sweep(glrm_s *h, double *hist_slot)
 {
     Scratch &s = h->s;
-    tmark(h, "reduce_stage1");
-    reduce_stage1<T><<<kRedBlocks, 256, 0, h->stream>>>(
+    tmark(h, "reduce");
+    reduce_kernel<T><<<reduce_blocks(2 * (h->m + h->n)), 256, 0, h->stream>>>(
         s.kept_obj_y, h->n, s.kept_reg_x, h->m, nullptr, 0, 0, T(0), nullptr, 0, 0, T(0), h->k,
-        s.acc_x, h->m, s.acc_y, h->n, s.red_part, s.red_cnt);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    tmark(h, "reduce_stage2");
-    reduce_stage2<<<1, 256, 0, h->stream>>>(s.red_part, s.red_cnt, kRedBlocks, hist_slot, s.accepts);
+        s.acc_x, h->m, s.acc_y, h->n, s.red_part, s.red_cnt, s.ticket, hist_slot, s.accepts);
     tmark(h, nullptr);
-    h->launches += 2;
+    h->launches += 1;
     return cudaGetLastError();
 }
 
@@ -721,15 +921,12 @@ cudaError_t Engine<T>::objective_at(glrm_s *h, const T *X, const T *Yt, double *
     cudaError_t e = dispatch_pass<T, true, false>(h->csr, X, Yt, h->k, loss_of<T>(h), nullptr,
                                                   s.part_loss, h->stream, nullptr, 0, (const T *)h->lscale);
     if (e != cudaSuccess) return e;
-    tmark(h, "reduce_stage1");
-    reduce_stage1<T><<<kRedBlocks, 256, 0, h->stream>>>(
+    tmark(h, "reduce");
+    reduce_kernel<T><<<reduce_blocks(h->csr.nchunks + (h->m + h->n) * h->k), 256, 0, h->stream>>>(
         s.part_loss, h->csr.nchunks, nullptr, 0, X, h->m, reg_code(h, true), (T)h->rx_w, Yt, h->n,
-        reg_code(h, false), (T)h->ry_w, h->k, nullptr, 0, nullptr, 0, s.red_part, s.red_cnt);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    tmark(h, "reduce_stage2");
-    reduce_stage2<<<1, 256, 0, h->stream>>>(s.red_part, s.red_cnt, kRedBlocks, out, nullptr);
+        reg_code(h, false), (T)h->ry_w, h->k, nullptr, 0, nullptr, 0, s.red_part, s.red_cnt, s.ticket, out, nullptr);
     tmark(h, nullptr);
-    h->launches += 2 + (h->csr.nchunks ? 1 : 0);
+    h->launches += 1 + (h->csr.nchunks ? 1 : 0);
     return cudaGetLastError();
 }
 

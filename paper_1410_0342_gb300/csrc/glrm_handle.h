@@ -81,6 +81,7 @@ struct Scratch {
     int32_t *acc_x = nullptr, *acc_y = nullptr;                  // m, n
     double *red_part = nullptr;     // kRedBlocks partial sums
     long long *red_cnt = nullptr;   // kRedBlocks x 2 partial counts
+    unsigned *ticket = nullptr;     // finished blocks of the running reduction (0 between launches)
     double *hist = nullptr;         // hist_cap objective history
     long long *accepts = nullptr;   // 2
     double *scalar = nullptr;       // 1
