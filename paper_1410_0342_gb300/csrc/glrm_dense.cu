@@ -53,11 +53,10 @@ constexpr int kDnRows = 128;     // own rows per CTA (UMMA M)
 constexpr int kDnWarps = 16;     // evaluating warp w: TMEM lanes 32 (w % 4) .. + 31, chunk columns 16 (w / 4) .. + 15
 constexpr int kDnThreads = (kDnWarps + 3) * 32;  // + the GEMM1 warp, the copy warp, the GEMM2 warp
 // TMEM columns: U at [0, 64) and [64, 128), two buffers of R (hi, mid, lo; 32
-// columns each) at [128, 224) and [224, 320), G from 320 (one block of KP
-// columns per part of W that gets its own accumulator, see DnG), the own rows
-// (hi, mid, lo; KP / 2 columns each) behind it
+// columns each) at [128, 224) and [224, 320), G at [320, 320 + KP), the own
+// rows (hi, mid, lo; KP / 2 columns each) from 384
 constexpr int kDnTmem = 512;
-constexpr int kDnColR = 128, kDnColG = 320;
+constexpr int kDnColR = 128, kDnColG = 320, kDnColOwn = 384;
 constexpr int kDnMaxStages = 4;
 
 // Column loss with its parameters in FP32 (kind as int bits, Huber
@@ -80,20 +79,6 @@ struct DenseArgs {
     float *part_grad;     // slots x k
     double *part_loss;    // slots
     int *err;
-};
-
-// GEMM2's accumulator blocks.  An MMA costs the tensor pipe the same from
-// N = 16 up to about N = 128 (44 cycles on an idle SM, measured), so the six
-// products R.part x W.part of a 16-row K step are issued as three MMAs with
-// W's parts side by side in N: R.hi x [hi | mid | lo], R.mid x [hi | mid] and
-// R.lo x [hi], each W part with its own KP columns of G, added at the end.
-// For KP = 64 that would take 192 columns, more than tensor memory has left:
-// there the hi and mid parts are separate MMAs into one block.
-template <int KP>
-struct DnG {
-    static constexpr int NB = KP <= 32 ? 3 : 1;  // blocks
-    static constexpr int Own = kDnColG + NB * KP;
-    static_assert(Own + 3 * KP / 2 <= kDnTmem, "tensor memory");
 };
 
 // Dynamic shared memory of one CTA: the A stages first (1024-byte aligned for
@@ -198,6 +183,45 @@ __device__ __forceinline__ unsigned long long ceil2(unsigned long long a)
 __device__ __forceinline__ bool whole_deriv(int kind, float lev)
 {
     return kind == kLossHinge || kind == kLossL1 || (kind == kLossOrdinal && lev <= 257.f);
+}
+
+// The logistic entries of a mixed block, with the scalar functions the X-step
+// of mixed columns uses; a loop over copies in local memory, so that this rare
+// path takes no registers from the others.
+__device__ __forceinline__ void dn_block_loop(const float (&u)[16], const float (&a)[16], float (&rr)[16], float &lsum)
+{
+    float uu[16], aa[16];
+#pragma unroll
+    for (int w = 0; w < 16; ++w) {
+        uu[w] = u[w];
+        aa[w] = a[w];
+    }
+#pragma unroll 1
+    for (int w = 0; w < 16; ++w) {
+        const bool v = aa[w] == aa[w];
+        float L;
+        const float d = loss_deriv_k<kLossLogistic, float>(uu[w], aa[w], 0.f, 0.f, L);
+        lsum += v ? L : 0.f;
+        uu[w] = v ? d : 0.f;
+    }
+#pragma unroll
+    for (int w = 0; w < 16; ++w) rr[w] = uu[w];
+}
+
+// The losses and derivatives of the scalar functions the sparse paths use,
+// for kinds without a packed form.
+template <int KIND>
+__device__ __forceinline__ void dn_block_plain(const float (&u)[16], const float (&a)[16], float prm, float lev,
+                                               float (&rr)[16], float &lsum)
+{
+#pragma unroll
+    for (int w = 0; w < 16; ++w) {
+        const bool v = a[w] == a[w];
+        float L;
+        const float d = loss_deriv_k<KIND, float>(u[w], a[w], prm, lev, L);
+        lsum += v ? L : 0.f;
+        rr[w] = v ? d : 0.f;
+    }
 }
 
 // Losses and derivatives of 16 entries that all lie inside the table and
@@ -327,14 +351,7 @@ __device__ __forceinline__ void dn_block(const float (&u)[16], const float (&a)[
             upk2(q, rr[w], rr[w + 1]);
         }
     } else {
-#pragma unroll
-        for (int w = 0; w < 16; ++w) {
-            const bool v = !MISS || a[w] == a[w];
-            float L;
-            const float d = loss_deriv_k<KIND, float>(u[w], a[w], prm, lev, L);
-            lsum += v ? L : 0.f;
-            rr[w] = v ? d : 0.f;
-        }
+        dn_block_plain<KIND>(u, a, prm, lev, rr, lsum);
     }
     float l0, l1;
     upk2(acc, l0, l1);
@@ -593,9 +610,9 @@ dense_pass_kernel(const DenseArgs p, const __grid_constant__ CUtensorMap amap)
                 mv[w / 2] = bf2_bits(__halves2bfloat162(m0, m1));
                 lv[w / 2] = bf2_bits(__halves2bfloat162(l0, l1));
             }
-            tmem_st8(taddr + lane_base + (uint32_t)(DnG<KP>::Own + c0 / 2), hv);
-            tmem_st8(taddr + lane_base + (uint32_t)(DnG<KP>::Own + KP / 2 + c0 / 2), mv);
-            tmem_st8(taddr + lane_base + (uint32_t)(DnG<KP>::Own + KP + c0 / 2), lv);
+            tmem_st8(taddr + lane_base + (uint32_t)(kDnColOwn + c0 / 2), hv);
+            tmem_st8(taddr + lane_base + (uint32_t)(kDnColOwn + KP / 2 + c0 / 2), mv);
+            tmem_st8(taddr + lane_base + (uint32_t)(kDnColOwn + KP + c0 / 2), lv);
         }
         tmem_wait_st();
     }
@@ -605,10 +622,11 @@ dense_pass_kernel(const DenseArgs p, const __grid_constant__ CUtensorMap amap)
 
     if (producer) {
         const bool lead = elect_one();  // the lane that issues
+        // (own or R part, W part) of the six products, smallest first; hi . hi last
+        constexpr int pa[6] = {1, 0, 2, 0, 1, 0};
+        constexpr int pb[6] = {1, 2, 0, 1, 0, 0};
         if (warp == kDnWarps && lead) {
-            // GEMM1 warp.  (own part, W part), smallest products first; hi . hi last
-            constexpr int pa[6] = {1, 0, 2, 0, 1, 0};
-            constexpr int pb[6] = {1, 2, 0, 1, 0, 0};
+            // GEMM1 warp
             for (int c = 0; ok && c < nq; ++c) {
                 const int s = c % 3, b = c & 1;
                 // U of chunk c - 2 is in registers, W's parts of chunk c are in
@@ -624,7 +642,7 @@ dense_pass_kernel(const DenseArgs p, const __grid_constant__ CUtensorMap amap)
 #pragma unroll
                     for (int ks = 0; ks < KP / 16; ++ks)
                         umma_bf16_ta(taddr + (uint32_t)(b * kDnNT),
-                                     taddr + (uint32_t)(DnG<KP>::Own + pa[pr] * (KP / 2) + ks * 8),
+                                     taddr + (uint32_t)(kDnColOwn + pa[pr] * (KP / 2) + ks * 8),
                                      d0 + ((pb[pr] * SM::pk + ks * 32) >> 4), idesc, pr > 0 || ks > 0);
                 umma_commit(&barG1[b]);
                 ++g1_issued;
@@ -645,33 +663,23 @@ dense_pass_kernel(const DenseArgs p, const __grid_constant__ CUtensorMap amap)
                 tc_fence_after();
                 const uint64_t d0 = umma_desc_sw(ptst + s * 3 * SM::pt, 2 * kDnNT);
                 const uint32_t r0 = taddr + (uint32_t)(kDnColR + (c & 1) * 96);
-                // the four warps of each 16 chunk columns say whether R has lower parts there
+                // the four warps of each 16 chunk columns say whether R has
+                // lower parts there: MMAs over zeros are left out (half of
+                // them on a table of Boolean and ordinal columns)
                 uint32_t wh[4];
                 *reinterpret_cast<uint4 *>(wh) = *reinterpret_cast<const uint4 *>(whole_s[c & 3]);
+                constexpr uint32_t idesc = umma_idesc_bf16(kDnRows, KP);
+                constexpr int P0 = B16 ? 5 : 0;  // the BF16 form: hi . hi only
 #pragma unroll
-                for (int ks = 0; ks < kDnNT / 16; ++ks) {
-                    const uint64_t dk = d0 + ((ks * 32) >> 4);
-                    const uint32_t rk = r0 + ks * 8;
-                    if constexpr (B16) {  // the BF16 form: hi . hi only
-                        umma_bf16_ta(taddr + kDnColG, rk, dk, umma_idesc_bf16(kDnRows, KP), c > 0 || ks > 0);
-                    } else if constexpr (DnG<KP>::NB == 3) {
-                        umma_bf16_ta(taddr + kDnColG, rk, dk, umma_idesc_bf16(kDnRows, 3 * KP), c > 0 || ks > 0);
-                        if (wh[ks] != 0x01010101u) {
-                            umma_bf16_ta(taddr + kDnColG, rk + 32, dk, umma_idesc_bf16(kDnRows, 2 * KP), true);
-                            umma_bf16_ta(taddr + kDnColG, rk + 64, dk, umma_idesc_bf16(kDnRows, KP), true);
+                for (int pr = P0; pr < 6; ++pr)
+#pragma unroll
+                    for (int ks = 0; ks < kDnNT / 16; ++ks)
+                        if (pr == P0 && ks == 0) {  // the first MMA of chunk 0 sets G
+                            umma_bf16_ta(taddr + kDnColG, r0 + pa[pr] * 32, d0 + (pb[pr] * SM::pt >> 4), idesc, c > 0);
+                        } else if (pa[pr] == 0 || wh[ks] != 0x01010101u) {
+                            umma_bf16_ta(taddr + kDnColG, r0 + pa[pr] * 32 + ks * 8,
+                                         d0 + ((pb[pr] * SM::pt + ks * 32) >> 4), idesc, true);
                         }
-                    } else {
-                        constexpr uint32_t id = umma_idesc_bf16(kDnRows, KP);
-                        umma_bf16_ta(taddr + kDnColG, rk, dk + (2 * SM::pt >> 4), id, c > 0 || ks > 0);
-                        if (wh[ks] != 0x01010101u) {
-                            umma_bf16_ta(taddr + kDnColG, rk + 32, dk + (SM::pt >> 4), id, true);
-                            umma_bf16_ta(taddr + kDnColG, rk + 64, dk, id, true);
-                            umma_bf16_ta(taddr + kDnColG, rk + 32, dk, id, true);
-                        }
-                        umma_bf16_ta(taddr + kDnColG, rk, dk + (SM::pt >> 4), id, true);
-                        umma_bf16_ta(taddr + kDnColG, rk, dk, id, true);
-                    }
-                }
                 umma_commit(&barG2[c & 3]);
                 ++g2_issued;
             }
@@ -793,7 +801,10 @@ dense_pass_kernel(const DenseArgs p, const __grid_constant__ CUtensorMap amap)
                         // kind, the lanes of that kind
                         for (unsigned todo = wkinds; todo; todo &= todo - 1u) {
                             const int kd = __ffs((int)todo) - 1;
-                            if (kd == __float_as_int(myspec.x)) dn_block_kind<true>(kd, u, a, prm, lev, rr, lsum);
+                            if (kd == __float_as_int(myspec.x)) {
+                                if (kd == kLossLogistic) dn_block_loop(u, a, rr, lsum);
+                                else dn_block_kind<true>(kd, u, a, prm, lev, rr, lsum);
+                            }
                             __syncwarp();
                         }
                     }
@@ -877,13 +888,6 @@ dense_pass_kernel(const DenseArgs p, const __grid_constant__ CUtensorMap amap)
             for (int bb = 0; bb < KP / 16; ++bb) {
                 float v[16];
                 tmem_ld16(taddr + lane_base + (uint32_t)(kDnColG + 16 * bb), v);
-                if constexpr (DnG<KP>::NB == 3 && !B16) {  // the products with W's mid and lo parts
-                    float v1[16], v2[16];
-                    tmem_ld16(taddr + lane_base + (uint32_t)(kDnColG + KP + 16 * bb), v1);
-                    tmem_ld16(taddr + lane_base + (uint32_t)(kDnColG + 2 * KP + 16 * bb), v2);
-#pragma unroll
-                    for (int w = 0; w < 16; ++w) v[w] += v1[w] + v2[w];
-                }
                 if (own_ok) {
 #pragma unroll
                     for (int w = 0; w < 16; ++w)
