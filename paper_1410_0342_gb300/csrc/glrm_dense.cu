@@ -1200,16 +1200,25 @@ struct PlanRange {
     bool tail;  // a half of a split item: launched after the others
 };
 
-double list_schedule_end(const std::vector<double> &t, int slots)
+// End of a list schedule of the items on `slots` SMs, or the first end found
+// at or beyond `limit`.  A binary heap of the times at which the SMs are free.
+double list_schedule_end(const std::vector<double> &t, int slots, double limit)
 {
-    std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
-    for (int i = 0; i < slots; ++i) free_at.push(0.0);
+    std::vector<double> h(slots + 1, 0.0);
+    h[slots] = HUGE_VAL;
     double end = 0;
     for (double c : t) {
-        const double f = free_at.top() + c;
-        free_at.pop();
-        free_at.push(f);
+        const double f = h[0] + c;
         end = std::max(end, f);
+        if (end >= limit) return end;
+        int i = 0;  // the SM's new time sinks from the root
+        for (int u = 1; u < slots; u = 2 * i + 1) {
+            u += h[u + 1] < h[u];
+            if (h[u] >= f) break;
+            h[i] = h[u];
+            i = u;
+        }
+        h[i] = f;
     }
     return end;
 }
@@ -1249,42 +1258,52 @@ ItemPlan plan_items(int64_t nown, int64_t nother, int sms, const std::vector<dou
                 q = e;
             }
         }
-        order(v);
+        order(v.begin(), v.end());
         return v;
     };
-    // the last `s` items of the launch order split in two at the middle of their cost
+    // the last `s` items of the launch order split in two at the middle of their
+    // cost (those of one chunk stay whole), the halves after all others
+    std::vector<PlanRange> w;
     auto split = [&](const std::vector<PlanRange> &v, int64_t s) {
-        std::vector<PlanRange> w(v.begin(), v.end() - s);
+        w.assign(v.begin(), v.end() - s);
+        for (auto r = v.end() - s; r != v.end(); ++r)
+            if (r->q1 - r->q0 < 2) w.push_back(*r);
+        const int64_t whole = (int64_t)w.size();
         for (auto r = v.end() - s; r != v.end(); ++r) {
-            if (r->q1 - r->q0 < 2) {
-                w.push_back(*r);
-                continue;
-            }
+            if (r->q1 - r->q0 < 2) continue;
             const double goal = 0.5 * (pre[r->q0] + pre[r->q1]);
             int64_t e = std::lower_bound(pre.begin() + r->q0, pre.begin() + r->q1, goal) - pre.begin();
             e = std::max<int64_t>(r->q0 + 1, std::min<int64_t>(e, r->q1 - 1));
             w.push_back({r->tile, r->q0, e, true});
             w.push_back({r->tile, e, r->q1, true});
         }
-        order(w);
-        return w;
+        order(w.begin() + whole, w.end());
     };
-    auto finish_time = [&](const std::vector<PlanRange> &v) {
-        std::vector<double> t(v.size());
-        for (size_t i = 0; i < v.size(); ++i) t[i] = tile_cost[v[i].tile] * (pre[v[i].q1] - pre[v[i].q0]) + fill;
-        return list_schedule_end(t, sms);
+    std::vector<double> t;
+    auto finish_time = [&](const std::vector<PlanRange> &v, double limit) {
+        t.resize(v.size());
+        double sum = 0;
+        for (size_t i = 0; i < v.size(); ++i)
+            sum += t[i] = tile_cost[v[i].tile] * (pre[v[i].q1] - pre[v[i].q0]) + fill;
+        return sum >= limit * sms ? sum / sms : list_schedule_end(t, sms, limit);
     };
     const double per0 = total / (double)std::max<int64_t>(tiles, 4LL * sms);
     std::vector<PlanRange> best = build(per0);
     if ((int64_t)best.size() <= 64LL * sms) {  // beyond that the last wave is a small share
-        double best_end = finish_time(best);
+        double best_end = finish_time(best, HUGE_VAL);
+        std::vector<PlanRange> last;
         for (int f = 0; f <= 10; ++f) {
             const std::vector<PlanRange> v = build(per0 * (1.0 + 0.03 * f));
             const int64_t n = (int64_t)v.size();
+            if (std::equal(v.begin(), v.end(), last.begin(), last.end(), [](const PlanRange &a, const PlanRange &b) {
+                    return a.tile == b.tile && a.q0 == b.q0 && a.q1 == b.q1;
+                }))
+                continue;  // tiles of one part each, say, are those of every target
+            last = v;
             for (int g = 0; g <= 24; ++g) {
-                const std::vector<PlanRange> w = g ? split(v, n * g / 24) : v;
-                const double end = finish_time(w);
-                if (end < best_end * (1.0 - 1e-9)) {
+                split(v, n * g / 24);
+                const double limit = best_end * (1.0 - 1e-9), end = finish_time(w, limit);
+                if (end < limit) {
                     best_end = end;
                     best = w;
                 }
