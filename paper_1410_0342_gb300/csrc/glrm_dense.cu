@@ -1234,10 +1234,8 @@ ItemPlan plan_items(int64_t nown, int64_t nother, int sms, const std::vector<dou
     for (int64_t t = 0; t < tiles; ++t) total += tile_cost[t] * pre[nch];
     const double fill = 1.3 * total / (double)(tiles * nch);
     auto mid = [](const PlanRange &r) { return r.q0 + r.q1; };
-    auto order = [&](std::vector<PlanRange> &v) {
-        std::stable_sort(v.begin(), v.end(), [&](const PlanRange &a, const PlanRange &b) {
-            return a.tail != b.tail ? !a.tail : mid(a) < mid(b);
-        });
+    auto order = [&](std::vector<PlanRange>::iterator a, std::vector<PlanRange>::iterator b) {
+        std::stable_sort(a, b, [&](const PlanRange &u, const PlanRange &v) { return mid(u) < mid(v); });
     };
     // the tile's chunks in np ranges of about equal cost, at least one chunk each
     auto build = [&](double per_item) {
@@ -1559,7 +1557,7 @@ cudaError_t dense_half_step(glrm_s *h, bool xstep)
     if (e != cudaSuccess) return e;
     tmark(h, xstep ? "prox_x" : "prox_y");
     e = launch_prox<float>(nseg, segchunk, (const float *)s.part_grad, s.part_loss, F, alpha, h->k, rk, rw,
-                           (float *)s.cand, s.f_old, s.r_old, s.r_new, st);
+                           (float *)s.cand, s.f_old, s.r_old, s.r_new, st, xstep ? h->dn.slots_x : h->dn.slots_y);
     if (e != cudaSuccess) return e;
     tmark(h, xstep ? "dense_loss_x" : "dense_loss_y");
     e = xstep ? launch_dense<true, false>(h, (const float *)s.cand, nullptr, s.part_loss2)
@@ -1600,19 +1598,18 @@ cudaError_t dense_grad_at(glrm_s *h, const float *X, const float *Yt, float *GX,
     tmark(h, "dense_grad_x");
     if ((e = launch_dense<true, true>(h, X, (float *)s.part_grad, s.part_loss)) != cudaSuccess) return e;
     tmark(h, "grad_seg_x");
-    seg_grad_kernel<float><<<blocks_for(h->m, kWarpsPerBlock), kWarpsPerBlock * 32, 0, h->stream>>>(
-        h->m, h->dn.segchunk_x, (const float *)s.part_grad, X, h->k, reg_code(h, true), (float)h->rx_w, reg, scale, GX);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch_seg_grad<float>(h->m, h->dn.segchunk_x, (const float *)s.part_grad, X, h->k, reg_code(h, true),
+                                    (float)h->rx_w, reg, scale, GX, h->stream, h->dn.slots_x)) != cudaSuccess)
+        return e;
     if ((e = dense_pack(h, X, h->m)) != cudaSuccess) return e;
     tmark(h, "dense_grad_y");
     if ((e = launch_dense<false, true>(h, Yt, (float *)s.part_grad, s.part_loss)) != cudaSuccess) return e;
     tmark(h, "grad_seg_y");
-    seg_grad_kernel<float><<<blocks_for(h->n, kWarpsPerBlock), kWarpsPerBlock * 32, 0, h->stream>>>(
-        h->n, h->dn.segchunk_y, (const float *)s.part_grad, Yt, h->k, reg_code(h, false), (float)h->ry_w, reg, scale,
-        GYt);
+    e = launch_seg_grad<float>(h->n, h->dn.segchunk_y, (const float *)s.part_grad, Yt, h->k, reg_code(h, false),
+                               (float)h->ry_w, reg, scale, GYt, h->stream, h->dn.slots_y);
     tmark(h, nullptr);
     h->launches += 2;
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace glrm

@@ -254,6 +254,37 @@ pass_kernel(int64_t nchunks, const int4 *__restrict__ chunks, const int32_t *__r
     if (lane == 0) part_loss[c] = ls;
 }
 
+// Sums of S <= 8 values over the warp, every lane receiving all of them, with
+// 9 additions instead of the butterflies' 5 S (an FP64 addition of a warp holds
+// its scheduler's FP64 unit for 64 cycles): in the first three steps each lane
+// passes on half of its values and keeps the sums of the other half.  The
+// same pairs are added in the same order as in warp butterflies of distance
+// 1, 2, 4, 8, 16: the results are those, bit for bit.
+template <int S>
+__device__ __forceinline__ void warp_sum_vec(double (&g)[S])
+{
+    static_assert(S <= 8, "three halving steps");
+    const int lane = threadIdx.x & 31;
+    double v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = i < S ? g[i] : 0.0;
+#pragma unroll
+    for (int st = 0; st < 3; ++st) {
+        const bool up = (lane >> st) & 1;
+        const int half = 4 >> st;
+#pragma unroll
+        for (int i = 0; i < half; ++i) {
+            const double give = up ? v[i] : v[i + half], keep = up ? v[i + half] : v[i];
+            v[i] = keep + shfl_xor(give, 1 << st);
+        }
+    }
+    v[0] += shfl_xor(v[0], 8);
+    v[0] += shfl_xor(v[0], 16);
+#pragma unroll
+    for (int i = 0; i < S; ++i)
+        g[i] = __shfl_sync(0xffffffffu, v[0], ((i >> 2) & 1) | (((i >> 1) & 1) << 1) | ((i & 1) << 2));
+}
+
 // A whole half-step of segments that fit in one chunk, a warp per segment:
 // gradient pass, prox, loss pass of the candidate, decision.  The candidate's
 // coordinates stay in the lanes that hold the gradient's (every lane group
@@ -330,10 +361,14 @@ seg_kernel(int64_t nseg, const int32_t *__restrict__ ptr, const int32_t *__restr
         for (int c = 0; c < S; ++c) g[c] = fma(d, w[c], g[c]);
         if (gl == 0) lsum += L;
     }
+    if constexpr (std::is_same<T, double>::value && G == 1 && S <= 8) {
+        warp_sum_vec<S>(g);
+    } else {
 #pragma unroll
-    for (int c = 0; c < S; ++c) {
+        for (int c = 0; c < S; ++c) {
 #pragma unroll
-        for (int o = G; o < 32; o <<= 1) g[c] += shfl_xor(g[c], o);
+            for (int o = G; o < 32; o <<= 1) g[c] += shfl_xor(g[c], o);
+        }
     }
     const double fo_loss = warp_sum((double)lsum);
     // the candidate, in the lanes' own coordinates
@@ -451,6 +486,79 @@ prox_kernel(int64_t nseg, const int32_t *__restrict__ segchunk, const T *__restr
         cand[s * k + c] = xp;
         ro += reg1t<T>(rkc, rw, x);
         rn += reg1t<T>(rkc, rw, xp);
+    }
+    ro = warp_sum(ro);
+    rn = warp_sum(rn);
+    const double ls = seg_loss_sum(part_loss, cb, ce, lane);
+    if (lane == 0) {
+        f_old[s] = ls + ro;
+        r_old[s] = ro;
+        r_new[s] = rn;
+    }
+}
+
+// A segment's gradient coordinates lane and lane + 32 on warp 0 of a CTA.  All
+// warps bring the partials into shared memory, warp 0 adds them in slot order
+// (the sums of prox_kernel, bit for bit).  For the few, long segments of a
+// tall table (80 to 100 partials for each of 1,000 columns) one warp loading
+// as it added was a chain of memory latencies: prox_y 47 -> 12 us.
+constexpr int kWideValues = 4096;
+template <class T>
+__device__ __forceinline__ void wide_gradient(const T *__restrict__ part_grad, int cb, int ce, int k, T *sh, T (&g)[2])
+{
+    const int lane = threadIdx.x & 31, per = kWideValues / k;
+    g[0] = g[1] = T(0);
+    for (int q0 = cb; q0 < ce; q0 += per) {
+        const int cnt = min(per, ce - q0);
+        if (q0 > cb) __syncthreads();  // the previous batch is summed
+#pragma unroll 4
+        for (int i = threadIdx.x; i < cnt * k; i += kWarpsPerBlock * 32) sh[i] = part_grad[(int64_t)q0 * k + i];
+        __syncthreads();
+        if (threadIdx.x < 32) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int c = lane + 32 * h;
+                if (c < k) {
+                    int q = 0;
+                    if (q0 == cb) g[h] = sh[c], q = 1;
+#pragma unroll 8
+                    for (; q < cnt; ++q) g[h] += sh[q * k + c];
+                }
+            }
+        }
+    }
+}
+
+// Segments with this many partials or more on average take a CTA each.
+constexpr int64_t kWideSlots = 16;
+
+template <class T>
+__global__ void __launch_bounds__(kWarpsPerBlock * 32)
+prox_wide_kernel(const int32_t *__restrict__ segchunk, const T *__restrict__ part_grad,
+                 const double *__restrict__ part_loss, const T *__restrict__ F, const T *__restrict__ alpha, int k,
+                 int rkind, T rw, T *__restrict__ cand, double *__restrict__ f_old, double *__restrict__ r_old,
+                 double *__restrict__ r_new)
+{
+    __shared__ T sh[kWideValues];
+    const int lane = threadIdx.x & 31;
+    const int64_t s = blockIdx.x;
+    const int cb = segchunk[s], ce = segchunk[s + 1];
+    T g[2];
+    wide_gradient<T>(part_grad, cb, ce, k, sh, g);
+    if (threadIdx.x >= 32) return;
+    const T al = alpha[s];
+    T ro = T(0), rn = T(0);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int c = lane + 32 * h;
+        if (c < k) {
+            const T x = F[s * k + c];
+            const int rkc = reg_kind_at(rkind, c, k);
+            const T xp = prox1<T>(rkc, rw, al, x - al * g[h]);
+            cand[s * k + c] = xp;
+            ro += reg1t<T>(rkc, rw, x);
+            rn += reg1t<T>(rkc, rw, xp);
+        }
     }
     ro = warp_sum(ro);
     rn = warp_sum(rn);
@@ -582,9 +690,12 @@ constexpr int64_t kNarrowSegments = 32768;
 template <class T>
 cudaError_t launch_prox(int64_t nseg, const int32_t *segchunk, const T *part_grad, const double *part_loss,
                         const T *F, const T *alpha, int k, int rk, T rw, T *cand, double *f_old, double *r_old,
-                        double *r_new, cudaStream_t st)
+                        double *r_new, cudaStream_t st, int64_t slots)
 {
-    if (nseg >= kNarrowSegments && k <= 64) {
+    if (slots >= kWideSlots * nseg) {  // slots: partials in all
+        prox_wide_kernel<T><<<(unsigned)nseg, kWarpsPerBlock * 32, 0, st>>>(
+            segchunk, part_grad, part_loss, F, alpha, k, rk, rw, cand, f_old, r_old, r_new);
+    } else if (nseg >= kNarrowSegments && k <= 64) {
         if (k <= 16)
             prox_narrow_kernel<T, 4><<<(unsigned)((nseg * 4 + 255) / 256), 256, 0, st>>>(
                 nseg, segchunk, part_grad, part_loss, F, alpha, k, rk, rw, cand, f_old, r_old, r_new);
@@ -675,6 +786,16 @@ reduce_kernel(const double *__restrict__ a, int64_t na, const double *__restrict
     if (ca) { range(nca, lo, hi); for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) c1 += ca[i]; }
     if (cb) { range(ncb, lo, hi); for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) c2 += cb[i]; }
     block_sums();
+    if (gridDim.x == 1) {
+        if (threadIdx.x == 0) {
+            if (out) *out = sh[0];
+            if (cnt_out) {
+                cnt_out[0] = shc[0][0];
+                cnt_out[1] = shc[1][0];
+            }
+        }
+        return;
+    }
     if (threadIdx.x == 0) {
         part[blockIdx.x] = sh[0];
         cnt[2 * blockIdx.x] = shc[0][0];
@@ -703,11 +824,12 @@ reduce_kernel(const double *__restrict__ a, int64_t na, const double *__restrict
     }
 }
 
-// Blocks of a reduction over `items` values: one per 1,024 values, at most
-// kRedBlocks (a small table's sum is not spread over 304 blocks).
+// Blocks of a reduction over `items` values: one up to 4,096 values (no
+// partials, no counter), then one per 1,024, at most kRedBlocks.
 inline unsigned reduce_blocks(int64_t items)
 {
-    return (unsigned)std::max<int64_t>(1, std::min<int64_t>(kRedBlocks, (items + 1023) / 1024));
+    if (items <= 4096) return 1;
+    return (unsigned)std::min<int64_t>(kRedBlocks, (items + 1023) / 1024);
 }
 
 // Gradient of each segment: sum of its chunk partials (+ the regulariser's
@@ -733,6 +855,40 @@ seg_grad_kernel(int64_t nseg, const int32_t *__restrict__ segchunk, const T *__r
         if (reg) g += reg_grad1<T>(reg_kind_at(rkind, c, k), rw, F[s * k + c]);
         G[s * k + c] = sc * g;
     }
+}
+
+template <class T>
+__global__ void __launch_bounds__(kWarpsPerBlock * 32)
+seg_grad_wide_kernel(const int32_t *__restrict__ segchunk, const T *__restrict__ part_grad, const T *__restrict__ F,
+                     int k, int rkind, T rw, bool reg, const double *__restrict__ scale, T *__restrict__ G)
+{
+    __shared__ T sh[kWideValues];
+    const int64_t s = blockIdx.x;
+    T g[2];
+    wide_gradient<T>(part_grad, segchunk[s], segchunk[s + 1], k, sh, g);
+    if (threadIdx.x >= 32) return;
+    const T sc = scale ? (T)*scale : T(1);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int c = threadIdx.x + 32 * h;
+        if (c < k) {
+            if (reg) g[h] += reg_grad1<T>(reg_kind_at(rkind, c, k), rw, F[s * k + c]);
+            G[s * k + c] = sc * g[h];
+        }
+    }
+}
+
+template <class T>
+cudaError_t launch_seg_grad(int64_t nseg, const int32_t *segchunk, const T *part_grad, const T *F, int k, int rk, T rw,
+                            bool reg, const double *scale, T *G, cudaStream_t st, int64_t slots)
+{
+    if (slots >= kWideSlots * nseg)
+        seg_grad_wide_kernel<T><<<(unsigned)nseg, kWarpsPerBlock * 32, 0, st>>>(segchunk, part_grad, F, k, rk, rw, reg,
+                                                                               scale, G);
+    else
+        seg_grad_kernel<T><<<blocks_for(nseg, kWarpsPerBlock), kWarpsPerBlock * 32, 0, st>>>(
+            nseg, segchunk, part_grad, F, k, rk, rw, reg, scale, G);
+    return cudaGetLastError();
 }
 
 template <class T>
@@ -811,6 +967,24 @@ cudaError_t dispatch_pass(const Orient &o, const T *F, const WT *W, int k, const
     return cudaErrorInvalidValue;
 }
 
+// The passes of a handle's orientation.
+template <class T, bool XSTEP, bool GRAD>
+cudaError_t run_pass(glrm_s *h, const T *F, const T *W, T *part_grad, double *part_loss, const int32_t *sel = nullptr,
+                     int want = 0, const T *lsc = nullptr)
+{
+    return dispatch_pass<T, XSTEP, GRAD>(XSTEP ? h->csr : h->csc, F, W, h->k, loss_of<T>(h), part_grad, part_loss,
+                                         h->stream, sel, want, lsc);
+}
+
+// The BF16 form's gradient passes: the other factor's rows from a BF16 copy.
+template <bool XSTEP>
+cudaError_t run_pass_bf16(glrm_s *h, const float *F, const __nv_bfloat16 *W, float *part_grad, double *part_loss,
+                          const int32_t *sel = nullptr, int want = 0)
+{
+    return dispatch_pass<float, XSTEP, true, __nv_bfloat16>(XSTEP ? h->csr : h->csc, F, W, h->k, h->loss_f, part_grad,
+                                                            part_loss, h->stream, sel, want);
+}
+
 template <class T, int K, bool XSTEP>
 cudaError_t launch_seg(glrm_s *h, const Orient &o, T *F, const T *W, T *alpha, int rk, T rw)
 {
@@ -826,8 +1000,12 @@ cudaError_t launch_seg(glrm_s *h, const Orient &o, T *F, const T *W, T *alpha, i
             XSTEP ? s.kept_obj_x : s.kept_obj_y, XSTEP ? s.kept_reg_x : s.kept_reg_y, XSTEP ? s.acc_x : s.acc_y,
             (const T *)h->lscale);
     };
-    if (vec) go(seg_kernel<T, K, XSTEP, true>);
-    else go(seg_kernel<T, K, XSTEP, false>);
+    if constexpr (K % 4 == 0) {
+        if (vec) go(seg_kernel<T, K, XSTEP, true>);
+        else go(seg_kernel<T, K, XSTEP, false>);
+    } else {
+        go(seg_kernel<T, K, XSTEP, false>);
+    }
     h->launches += 1;
     return cudaGetLastError();
 }
@@ -839,6 +1017,10 @@ cudaError_t dispatch_seg(glrm_s *h, const Orient &o, T *F, const T *W, T *alpha,
 #define GLRM_SEG_CASE(KK) \
     if (k <= KK) return launch_seg<T, KK, XSTEP>(h, o, F, W, alpha, rk, rw);
     GLRM_SEG_CASE(4)
+    if constexpr (std::is_same<T, double>::value) {  // no padding through the FP64 unit at small ranks
+        GLRM_SEG_CASE(5)
+        GLRM_SEG_CASE(6)
+    }
     GLRM_SEG_CASE(8)
     GLRM_SEG_CASE(12)
     GLRM_SEG_CASE(16)
@@ -876,18 +1058,16 @@ cudaError_t Engine<T>::half_step(glrm_s *h, bool xstep)
     }
     tmark(h, xstep ? "pass_grad_x" : "pass_grad_y");
     const T *lsc = (const T *)h->lscale;
-    e = xstep ? dispatch_pass<T, true, true>(o, F, W, k, loss_of<T>(h), (T *)s.part_grad, s.part_loss, st, nullptr, 0, lsc)
-              : dispatch_pass<T, false, true>(o, F, W, k, loss_of<T>(h), (T *)s.part_grad, s.part_loss, st, nullptr, 0, lsc);
+    e = xstep ? run_pass<T, true, true>(h, F, W, (T *)s.part_grad, s.part_loss, nullptr, 0, lsc)
+              : run_pass<T, false, true>(h, F, W, (T *)s.part_grad, s.part_loss, nullptr, 0, lsc);
     if (e != cudaSuccess) return e;
     tmark(h, xstep ? "prox_x" : "prox_y");
     e = launch_prox<T>(o.nseg, o.segchunk, (const T *)s.part_grad, s.part_loss, F, alpha, k, rk, rw, (T *)s.cand,
-                       s.f_old, s.r_old, s.r_new, st);
+                       s.f_old, s.r_old, s.r_new, st, o.nchunks);
     if (e != cudaSuccess) return e;
     tmark(h, xstep ? "pass_loss_x" : "pass_loss_y");
-    e = xstep ? dispatch_pass<T, true, false>(o, (const T *)s.cand, W, k, loss_of<T>(h), nullptr, s.part_loss2, st,
-                                              nullptr, 0, lsc)
-              : dispatch_pass<T, false, false>(o, (const T *)s.cand, W, k, loss_of<T>(h), nullptr, s.part_loss2, st,
-                                               nullptr, 0, lsc);
+    e = xstep ? run_pass<T, true, false>(h, (const T *)s.cand, W, nullptr, s.part_loss2, nullptr, 0, lsc)
+              : run_pass<T, false, false>(h, (const T *)s.cand, W, nullptr, s.part_loss2, nullptr, 0, lsc);
     if (e != cudaSuccess) return e;
     tmark(h, xstep ? "decide_x" : "decide_y");
     e = launch_decide<T>(o.nseg, o.segchunk, s.part_loss2, s.f_old, s.r_old, s.r_new, (const T *)s.cand, F, alpha, k,
@@ -918,8 +1098,7 @@ cudaError_t Engine<T>::objective_at(glrm_s *h, const T *X, const T *Yt, double *
 {
     Scratch &s = h->s;
     tmark(h, "objective_pass");
-    cudaError_t e = dispatch_pass<T, true, false>(h->csr, X, Yt, h->k, loss_of<T>(h), nullptr,
-                                                  s.part_loss, h->stream, nullptr, 0, (const T *)h->lscale);
+    cudaError_t e = run_pass<T, true, false>(h, X, Yt, nullptr, s.part_loss, nullptr, 0, (const T *)h->lscale);
     if (e != cudaSuccess) return e;
     tmark(h, "reduce");
     reduce_kernel<T><<<reduce_blocks(h->csr.nchunks + (h->m + h->n) * h->k), 256, 0, h->stream>>>(
@@ -949,40 +1128,30 @@ cudaError_t Engine<T>::grad_at(glrm_s *h, const T *X, const T *Yt, T *GX, T *GYt
     }
     tmark(h, "grad_pass_x");
     if constexpr (std::is_same<T, float>::value) {
-        if (bf16)
-            e = dispatch_pass<T, true, true, __nv_bfloat16>(h->csr, X, s.yt_bf16, h->k, loss_of<T>(h),
-                                                            (T *)s.part_grad, s.part_loss, h->stream);
-        else
-            e = dispatch_pass<T, true, true>(h->csr, X, Yt, h->k, loss_of<T>(h), (T *)s.part_grad,
-                                             s.part_loss, h->stream, nullptr, 0, (const T *)h->lscale);
+        if (bf16) e = run_pass_bf16<true>(h, X, s.yt_bf16, (T *)s.part_grad, s.part_loss);
+        else e = run_pass<T, true, true>(h, X, Yt, (T *)s.part_grad, s.part_loss, nullptr, 0, (const T *)h->lscale);
     } else {
-        e = dispatch_pass<T, true, true>(h->csr, X, Yt, h->k, loss_of<T>(h), (T *)s.part_grad, s.part_loss,
-                                         h->stream, nullptr, 0, (const T *)h->lscale);
+        e = run_pass<T, true, true>(h, X, Yt, (T *)s.part_grad, s.part_loss, nullptr, 0, (const T *)h->lscale);
     }
     if (e != cudaSuccess) return e;
     tmark(h, "grad_seg_x");
-    seg_grad_kernel<T><<<blocks_for(h->m, kWarpsPerBlock), kWarpsPerBlock * 32, 0, h->stream>>>(
-        h->m, h->csr.segchunk, (const T *)s.part_grad, X, h->k, reg_code(h, true), (T)h->rx_w, reg, scale, GX);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch_seg_grad<T>(h->m, h->csr.segchunk, (const T *)s.part_grad, X, h->k, reg_code(h, true), (T)h->rx_w,
+                                reg, scale, GX, h->stream, h->csr.nchunks)) != cudaSuccess)
+        return e;
     tmark(h, "grad_pass_y");
     if constexpr (std::is_same<T, float>::value) {
-        if (bf16)
-            e = dispatch_pass<T, false, true, __nv_bfloat16>(h->csc, Yt, s.x_bf16, h->k, loss_of<T>(h),
-                                                             (T *)s.part_grad, s.part_loss, h->stream);
-        else
-            e = dispatch_pass<T, false, true>(h->csc, Yt, X, h->k, loss_of<T>(h), (T *)s.part_grad,
-                                              s.part_loss, h->stream, nullptr, 0, (const T *)h->lscale);
+        if (bf16) e = run_pass_bf16<false>(h, Yt, s.x_bf16, (T *)s.part_grad, s.part_loss);
+        else e = run_pass<T, false, true>(h, Yt, X, (T *)s.part_grad, s.part_loss, nullptr, 0, (const T *)h->lscale);
     } else {
-        e = dispatch_pass<T, false, true>(h->csc, Yt, X, h->k, loss_of<T>(h), (T *)s.part_grad,
-                                          s.part_loss, h->stream, nullptr, 0, (const T *)h->lscale);
+        e = run_pass<T, false, true>(h, Yt, X, (T *)s.part_grad, s.part_loss, nullptr, 0, (const T *)h->lscale);
     }
     if (e != cudaSuccess) return e;
     tmark(h, "grad_seg_y");
-    seg_grad_kernel<T><<<blocks_for(h->n, kWarpsPerBlock), kWarpsPerBlock * 32, 0, h->stream>>>(
-        h->n, h->csc.segchunk, (const T *)s.part_grad, Yt, h->k, reg_code(h, false), (T)h->ry_w, reg, scale, GYt);
+    e = launch_seg_grad<T>(h->n, h->csc.segchunk, (const T *)s.part_grad, Yt, h->k, reg_code(h, false), (T)h->ry_w, reg,
+                           scale, GYt, h->stream, h->csc.nchunks);
     tmark(h, nullptr);
     h->launches += 2 + (h->csr.nchunks ? 1 : 0) + (h->csc.nchunks ? 1 : 0);
-    return cudaGetLastError();
+    return e;
 }
 
 template <class T>
