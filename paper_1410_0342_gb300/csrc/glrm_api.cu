@@ -455,9 +455,10 @@ const char *flag_message(int f)
 }
 
 // Density from which an FP32 observed set is stored densely (NaN marking the
-// missing cells) and swept by the tensor-core form: the dense passes cost
-// about 13 ps per cell against about 30 ps per observed entry for the masked
-// sparse path (mixed table, k = 20, measured on GB300).
+// missing cells) and swept by the tensor-core form.  Below it the dense sweeps
+// are still the faster ones on large tables (50,021 x 701, k = 18, 25%: 414
+// against 850 us), but the split products' factors are further from the FP64
+// sweep's there than the sparse paths' (5.1e-7 against 5.2e-8 relative).
 constexpr double kDenseAutoDensity = 0.4;
 
 // Whether the observed set goes to the dense form: 1 yes, 0 no, else a
@@ -1082,6 +1083,9 @@ int glrm_create(int64_t m, int64_t n, int32_t k, const glrm_loss *col_loss, int3
     h->prec = precision;
     h->stream = (cudaStream_t)stream;
     h->loss_host = spec;
+    h->loss_uniform = std::all_of(spec.begin(), spec.end(), [&](const LossSpec &L) {
+        return L.kind == spec[0].kind && L.levels == spec[0].levels && L.param == spec[0].param;
+    });
     h->rx_kind = rx_kind;
     h->ry_kind = ry_kind;
     h->rx_w = rx_weight;

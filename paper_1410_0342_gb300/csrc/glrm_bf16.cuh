@@ -157,19 +157,17 @@ inline cudaError_t bf16_half_step(glrm_s *h, bool xstep)
     h->launches += 1;
     // gradient: BF16 rows for segments whose last step was accepted, FP32 rows for the others
     tmark(h, xstep ? "bf16_grad_x" : "bf16_grad_y");
-    e = xstep ? dispatch_pass<float, true, true, __nv_bfloat16>(o, F, Wb, k, h->loss_f, (float *)s.part_grad,
-                                                                  s.part_loss, st, acc, 1)
-              : dispatch_pass<float, false, true, __nv_bfloat16>(o, F, Wb, k, h->loss_f, (float *)s.part_grad,
-                                                                   s.part_loss, st, acc, 1);
+    e = xstep ? run_pass_bf16<true>(h, F, Wb, (float *)s.part_grad, s.part_loss, acc, 1)
+              : run_pass_bf16<false>(h, F, Wb, (float *)s.part_grad, s.part_loss, acc, 1);
     if (e != cudaSuccess) return e;
     tmark(h, xstep ? "fp32_grad_x" : "fp32_grad_y");
-    e = xstep ? dispatch_pass<float, true, true>(o, F, W, k, h->loss_f, (float *)s.part_grad, s.part_loss, st, acc, 0)
-              : dispatch_pass<float, false, true>(o, F, W, k, h->loss_f, (float *)s.part_grad, s.part_loss, st, acc, 0);
+    e = xstep ? run_pass<float, true, true>(h, F, W, (float *)s.part_grad, s.part_loss, acc, 0)
+              : run_pass<float, false, true>(h, F, W, (float *)s.part_grad, s.part_loss, acc, 0);
     if (e != cudaSuccess) return e;
     h->launches += 2 * (o.nchunks ? 1 : 0);
     tmark(h, xstep ? "prox_x" : "prox_y");
     e = launch_prox<float>(o.nseg, o.segchunk, (const float *)s.part_grad, s.part_loss, F, alpha, k, rk, rw,
-                           (float *)s.cand, s.f_old, s.r_old, s.r_new, st);
+                           (float *)s.cand, s.f_old, s.r_old, s.r_new, st, o.nchunks);
     if (e != cudaSuccess) return e;
     tmark(h, xstep ? "cand_x" : "cand_y");
     e = xstep ? cand_pass<true>(h, o, F, (const float *)s.cand, W) : cand_pass<false>(h, o, F, (const float *)s.cand, W);

@@ -981,6 +981,7 @@ template <bool XSTEP>
 cudaError_t run_pass_bf16(glrm_s *h, const float *F, const __nv_bfloat16 *W, float *part_grad, double *part_loss,
                           const int32_t *sel = nullptr, int want = 0)
 {
+    if (staged_bf16_ok(h->k, W)) return staged_pass_bf16(h, XSTEP, F, W, part_grad, part_loss, sel, want);
     return dispatch_pass<float, XSTEP, true, __nv_bfloat16>(XSTEP ? h->csr : h->csc, F, W, h->k, h->loss_f, part_grad,
                                                             part_loss, h->stream, sel, want);
 }

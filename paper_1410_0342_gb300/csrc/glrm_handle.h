@@ -163,6 +163,7 @@ struct glrm_s {
     cudaStream_t stream = nullptr;
     std::vector<glrm::LossSpec> loss_host;
     glrm::LossSpec *loss_dev = nullptr;
+    bool loss_uniform = false;  // every column has the same loss
     glrm::LossSpecF *loss_f = nullptr;  // the same losses with FP32 parameters (FP32 kernels)
     int rx_kind = 0, ry_kind = 0;
     bool offset = false;  // last coordinate of X held at 1, of Y unpenalised (glrm_set_offset)
@@ -265,6 +266,10 @@ cudaError_t launch_check_entries(const Orient &o, bool rows, int64_t other, int6
                                  const LossSpec *loss, int *flag, unsigned long long *digest, cudaStream_t st);
 cudaError_t launch_digest_compare(const unsigned long long *d, int *flag, cudaStream_t st);
 cudaError_t bf16_half_step_entry(glrm_s *h, bool xstep);
+// The BF16 form's gradient pass of large ranks through shared memory (glrm_staged.cu).
+bool staged_bf16_ok(int k, const void *W);
+cudaError_t staged_pass_bf16(glrm_s *h, bool xstep, const float *F, const __nv_bfloat16 *W, float *pg, double *pl,
+                             const int32_t *sel, int want);
 cudaError_t launch_fill_i32(int32_t *p, int64_t n, int32_t v, cudaStream_t st);
 // Per-column statistics mu_j, sigma2_j of the loss scaling (glrm_stats.cu).
 cudaError_t launch_column_stats(glrm_s *h, double *mu, double *s2);
