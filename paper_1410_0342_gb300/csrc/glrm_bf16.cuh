@@ -27,12 +27,13 @@ namespace glrm {
 
 // The candidate pass: per chunk, the losses at the segment's current factor
 // f and at its candidate f+ from one gather of each other-factor row (FP32).
-template <int K, bool XSTEP, bool VEC>
+template <int K, bool XSTEP, int VEC>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
 cand_pass_kernel(int64_t nchunks, const int4 *__restrict__ chunks, const int32_t *__restrict__ order,
                  const int32_t *__restrict__ idx, const float *__restrict__ val, const float *__restrict__ F,
                  const float *__restrict__ C, const float *__restrict__ W, int k,
-                 const LossSpecF *__restrict__ loss, double *__restrict__ part_old, double *__restrict__ part_new)
+                 const LossSpecF *__restrict__ loss, double *__restrict__ part_old, double *__restrict__ part_new,
+                 bool uni)
 {
     using LN = Lanes<K>;
     constexpr int G = LN::G, S = LN::S, PER = LN::PER, VW = 4;
@@ -47,22 +48,33 @@ cand_pass_kernel(int64_t nchunks, const int4 *__restrict__ chunks, const int32_t
     load_lane<float, S, G, VW, VEC>(fp, C + (int64_t)ch.x * k, gl, k);
     float lo = 0.f, ln = 0.f;
     LossSpecF sp;
-    if constexpr (!XSTEP) sp = loss[ch.x];
+    sp = loss[XSTEP ? 0 : ch.x];  // of every column, when uni
     // software pipeline as in the loss passes: the next group's index,
-    // value, loss and row are loaded before the current group is evaluated
-    float an = 0.f, wn[S];
+    // value, loss and row are loaded before the current group is evaluated,
+    // index and value one group earlier still
+    int jn = 0;
+    float an = 0.f, an2 = 0.f, wn[S];
     LossSpecF spn = sp;
+    auto ahead = [&](int e) {
+        if (e < ch.z) {
+            jn = __ldg(idx + e);
+            an2 = __ldg(val + e);
+        }
+    };
     auto fetch = [&](int e) {
         if (e < ch.z) {
-            const int jn = __ldg(idx + e);
-            an = __ldg(val + e);
+            an = an2;
             load_lane<float, S, G, VW, VEC>(wn, W + (int64_t)jn * k, gl, k);
-            if constexpr (XSTEP) spn = loss[jn];
+            if constexpr (XSTEP) {
+                if (!uni) spn = loss[jn];
+            }
+            ahead(e + PER);
         } else {
 #pragma unroll
             for (int s = 0; s < S; ++s) wn[s] = 0.f;
         }
     };
+    ahead(ch.y + grp);
     fetch(ch.y + grp);
     for (int base = ch.y; base < ch.z; base += PER) {
         const bool ok = base + grp < ch.z;
@@ -91,7 +103,8 @@ cand_pass_kernel(int64_t nchunks, const int4 *__restrict__ chunks, const int32_t
             ln += L1;
         }
     }
-    const double so = warp_sum((double)lo), sn = warp_sum((double)ln);
+    double so, sn;
+    warp_sum_two((double)lo, (double)ln, so, sn);
     if (lane == 0) {
         part_old[c] = so;
         part_new[c] = sn;
@@ -108,10 +121,10 @@ cudaError_t launch_cand(glrm_s *h, const Orient &o, const float *F, const float 
     const unsigned nb = blocks_for(o.nchunks, kWarpsPerBlock);
     auto go = [&](auto kern) {
         kern<<<nb, kWarpsPerBlock * 32, 0, h->stream>>>(o.nchunks, o.chunks, o.order, o.idx, (const float *)o.val, F, C,
-                                                        W, k, h->loss_f, h->s.part_loss, h->s.part_loss2);
+                                                        W, k, h->loss_f, h->s.part_loss, h->s.part_loss2, h->loss_uniform);
     };
-    if (vec) go(cand_pass_kernel<K, XSTEP, true>);
-    else go(cand_pass_kernel<K, XSTEP, false>);
+    if (vec) go(cand_pass_kernel<K, XSTEP, kUnits>);
+    else go(cand_pass_kernel<K, XSTEP, kScalar>);
     h->launches += 1;
     return cudaGetLastError();
 }

@@ -41,18 +41,29 @@ struct Lanes {
 // ...: at every load instruction the G lanes of an entry read G adjacent
 // units, whole 32-byte sectors of the row, so each sector is fetched once.
 // Slot s of lane gl holds coordinate VW ((s / VW) G + gl) + s % VW.  The
-// scalar form (any k) gives lane gl the contiguous coordinates gl S .. gl S + S - 1.
-template <int S, int G, int VW, bool VEC>
+// scalar form (any k) gives lane gl the contiguous coordinates gl S .. gl S + S - 1;
+// where one lane holds a whole FP32 row of even k it reads them in pairs.
+constexpr int kScalar = 0, kUnits = 1, kPairs = 2;
+
+template <int S, int G, int VW, int VEC>
 __device__ __forceinline__ int slot_coord(int s, int gl)
 {
-    return VEC ? VW * ((s / VW) * G + gl) + s % VW : gl * S + s;
+    return VEC == kUnits ? VW * ((s / VW) * G + gl) + s % VW : gl * S + s;
 }
 
 // A row's slots for lane gl in the layout above (T values, units of VW).
-template <class T, int S, int G, int VW, bool VEC>
+template <class T, int S, int G, int VW, int VEC>
 __device__ __forceinline__ void load_lane(T (&v)[S], const T *__restrict__ row, int gl, int k)
 {
-    if constexpr (VEC) {
+    if constexpr (VEC == kPairs) {
+        static_assert(G == 1 && S % 2 == 0 && sizeof(T) == 4, "pairs are of whole FP32 rows");
+#pragma unroll
+        for (int q = 0; q < S / 2; ++q) {
+            const float2 t = 2 * q < k ? __ldg(reinterpret_cast<const float2 *>(row) + q) : make_float2(0.f, 0.f);
+            v[2 * q] = t.x;
+            v[2 * q + 1] = t.y;
+        }
+    } else if constexpr (VEC == kUnits) {
         constexpr int VT = 16 / (int)sizeof(T);  // values per 16-byte load
         static_assert(S % VW == 0 && VW % VT == 0, "slots must be whole units");
 #pragma unroll
@@ -80,11 +91,11 @@ __device__ __forceinline__ void load_lane(T (&v)[S], const T *__restrict__ row, 
 }
 
 // The same for a BF16 row (units of 8 values), widened to FP32.
-template <int S, int G, bool VEC>
+template <int S, int G, int VEC>
 __device__ __forceinline__ void load_lane_bf16(float (&v)[S], const __nv_bfloat16 *__restrict__ row, int gl,
                                                int k)
 {
-    if constexpr (VEC) {
+    if constexpr (VEC == kUnits) {
         static_assert(S % 8 == 0, "bf16 slots must be whole units");
 #pragma unroll
         for (int q = 0; q < S / 8; ++q) {
@@ -102,16 +113,26 @@ __device__ __forceinline__ void load_lane_bf16(float (&v)[S], const __nv_bfloat1
     }
 }
 
+// Rows that one lane holds whole may be read in pairs (even k, 8-byte aligned).
+template <class WT, int K>
+constexpr bool pairs_ok = std::is_same<WT, float>::value && Lanes<K>::G == 1;
+
 // Coordinates per 16-byte unit of a row of type WT.
 template <class WT>
 constexpr int unit_of() { return 16 / (int)sizeof(WT); }
 
-template <class T, int S, int G, bool VEC, class WT>
+template <class T, int S, int G, int VEC, class WT>
 __device__ __forceinline__ void load_lane_w(T (&v)[S], const WT *__restrict__ row, int gl, int k)
 {
     if constexpr (std::is_same<WT, __nv_bfloat16>::value) load_lane_bf16<S, G, VEC>(v, row, gl, k);
     else load_lane<T, S, G, unit_of<WT>(), VEC>(v, row, gl, k);
 }
+
+// Whether a block's loss sums go through one warp: an FP64 addition holds a
+// scheduler's FP64 unit for 64 cycles, so the five of each chunk's butterfly
+// were some 16 of 86 us for the 60,000 short rows of a ratings table.
+template <class T>
+constexpr bool kBlockSums = std::is_same<T, float>::value;
 
 // One warp per chunk: entries base + grp for base = begin, begin + PER, ...
 // (G lanes per entry, PER = 32 / G entries per iteration), the rows of the
@@ -119,25 +140,40 @@ __device__ __forceinline__ void load_lane_w(T (&v)[S], const WT *__restrict__ ro
 // chunk launch order; with `sel` (nullable) the launch takes only the chunks
 // of segments whose sel value is nonzero exactly when want is.  `lsc`
 // (nullable) holds per-column loss weights: entry (i, j) contributes
-// lsc[j] L_j and lsc[j] L_j' (the scaled losses of Section 4.3).
-template <class T, int K, bool XSTEP, bool VEC, bool GRAD, class WT = T>
+// lsc[j] L_j and lsc[j] L_j' (the scaled losses of Section 4.3).  uni: all
+// columns have one loss, read once instead of gathered with each entry.
+//
+// Bound by the gathers: their latency (index, then row) and, at k = 64, L1's
+// rate.  An entry's index and value are loaded a group ahead of its row, so
+// that one latency is exposed instead of two; rows are read in the widest
+// units their rank and address allow.  Completion table (1,000,000 x 20,000,
+// 200 a row, k = 64), columns: gradient 5.0 -> 3.7 ms, loss 3.2 -> 3.0 ms;
+// 60,013 x 5,003 ratings, k = 10: 86 -> 62, 68 -> 44 and 70 -> 49 us.
+template <class T, int K, bool XSTEP, int VEC, bool GRAD, class WT = T>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
 pass_kernel(int64_t nchunks, const int4 *__restrict__ chunks, const int32_t *__restrict__ order,
             const int32_t *__restrict__ idx, const T *__restrict__ val, const T *__restrict__ F,
             const WT *__restrict__ W, int k, const LossOf<T> *__restrict__ loss, T *__restrict__ part_grad,
             double *__restrict__ part_loss, const int32_t *__restrict__ sel, int want,
-            const T *__restrict__ lsc)
+            const T *__restrict__ lsc, bool uni)
 {
     using LN = Lanes<K>;
     constexpr int G = LN::G, S = LN::S, PER = LN::PER;
     constexpr int VW = unit_of<WT>();  // f and the gathered rows share the layout of WT's units
     const int lane = threadIdx.x & 31;
     const int64_t lin = (int64_t)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
-    if (lin >= nchunks) return;  // the whole warp leaves together
-    const int64_t c = order ? (int64_t)__ldg(order + lin) : lin;
     const int gl = lane % G, grp = lane / G;
-    const int4 ch = chunks[c];
-    if (sel && ((__ldg(sel + ch.x) != 0) != (want != 0))) return;  // another launch takes this segment
+    int64_t c = -1;
+    int4 ch = make_int4(0, 0, 0, 0);
+    if (lin < nchunks) {
+        c = order ? (int64_t)__ldg(order + lin) : lin;
+        ch = chunks[c];
+        if (sel && ((__ldg(sel + ch.x) != 0) != (want != 0))) c = -1;  // another launch takes this segment
+    }
+    if constexpr (!kBlockSums<T>) {
+        if (c < 0) return;  // the whole warp leaves together
+    }
+    if (c < 0) ch.z = ch.y;
     T f[S], g[S];
     load_lane<T, S, G, VW, VEC>(f, F + (int64_t)ch.x * k, gl, k);
 #pragma unroll
@@ -145,36 +181,46 @@ pass_kernel(int64_t nchunks, const int4 *__restrict__ chunks, const int32_t *__r
     T lsum = T(0);
     LossOf<T> sp;
     T wsc = T(1);
-    if constexpr (!XSTEP) {
+    if constexpr (XSTEP) {
+        sp = loss[0];  // of every column, when uni
+    } else {
         sp = loss[ch.x];
         if (lsc) wsc = __ldg(lsc + ch.x);
     }
     if constexpr (!GRAD) {
         // loss passes: a software pipeline, the next group of entries' index,
         // value, loss and gathered row loaded before the current group is
-        // evaluated (two gathers per lane in flight).  The gradient passes
+        // evaluated (two gathers per lane in flight), its index and value one
+        // group before that (the row's address waits on them).  The gradient passes
         // keep one: their gradient registers would cut the occupancy more
         // than the second gather gains (94 against 73 registers, measured
         // slower on the k = 64 completion table).
         int jn = 0;
-        T an = T(0);
+        T an = T(0), an2 = T(0);
         T wn[S];
         LossOf<T> spn = sp;
         T wscn = wsc;
-        auto fetch = [&](int e) {
+        auto ahead = [&](int e) {
             if (e < ch.z) {
                 jn = __ldg(idx + e);
-                an = __ldg(val + e);
+                an2 = __ldg(val + e);
+            }
+        };
+        auto fetch = [&](int e) {
+            if (e < ch.z) {
+                an = an2;
                 load_lane_w<T, S, G, VEC, WT>(wn, W + (int64_t)jn * k, gl, k);
                 if constexpr (XSTEP) {
-                    spn = loss[jn];
+                    if (!uni) spn = loss[jn];
                     if (lsc) wscn = __ldg(lsc + jn);
                 }
+                ahead(e + PER);
             } else {
 #pragma unroll
                 for (int s = 0; s < S; ++s) wn[s] = T(0);
             }
         };
+        ahead(ch.y + grp);
         fetch(ch.y + grp);
         for (int base = ch.y; base < ch.z; base += PER) {
             const bool ok = base + grp < ch.z;
@@ -200,15 +246,24 @@ pass_kernel(int64_t nchunks, const int4 *__restrict__ chunks, const int32_t *__r
             }
         }
     } else {
+        // the next group's index and value are on their way while the row waits
+        int jn = 0;
+        T an = T(0);
+        if (ch.y + grp < ch.z) {
+            jn = __ldg(idx + ch.y + grp);
+            an = __ldg(val + ch.y + grp);
+        }
         for (int base = ch.y; base < ch.z; base += PER) {
             const int e = base + grp;
             const bool ok = e < ch.z;
-            int j = 0;
-            T a = T(0);
+            const int j = jn;
+            const T a = an;
+            if (e + PER < ch.z) {
+                jn = __ldg(idx + e + PER);
+                an = __ldg(val + e + PER);
+            }
             T w[S];
             if (ok) {
-                j = __ldg(idx + e);
-                a = __ldg(val + e);
                 load_lane_w<T, S, G, VEC, WT>(w, W + (int64_t)j * k, gl, k);
             } else {
 #pragma unroll
@@ -221,7 +276,7 @@ pass_kernel(int64_t nchunks, const int4 *__restrict__ chunks, const int32_t *__r
             for (int o = 1; o < G; o <<= 1) u += shfl_xor(u, o);
             if (ok) {
                 if constexpr (XSTEP) {
-                    sp = loss[j];
+                    if (!uni) sp = loss[j];
                     if (lsc) wsc = __ldg(lsc + j);
                 }
                 T L;
@@ -242,7 +297,7 @@ pass_kernel(int64_t nchunks, const int4 *__restrict__ chunks, const int32_t *__r
 #pragma unroll
             for (int o = G; o < 32; o <<= 1) g[s] += shfl_xor(g[s], o);
         }
-        if (grp == 0) {
+        if (grp == 0 && c >= 0) {
 #pragma unroll
             for (int s = 0; s < S; ++s) {
                 const int cc = slot_coord<S, G, VW, VEC>(s, gl);
@@ -250,8 +305,26 @@ pass_kernel(int64_t nchunks, const int4 *__restrict__ chunks, const int32_t *__r
             }
         }
     }
-    const double ls = warp_sum((double)lsum);
-    if (lane == 0) part_loss[c] = ls;
+    if constexpr (kBlockSums<T>) {
+        // the block's loss sums in one warp: 8 of a chunk's 32 terms a lane,
+        // 9 FP64 additions of one warp for the block instead of 5 of each warp
+        __shared__ float sh[kWarpsPerBlock][33];
+        __shared__ int64_t shc[kWarpsPerBlock];
+        sh[threadIdx.x >> 5][lane] = lsum;
+        if (lane == 0) shc[threadIdx.x >> 5] = c;
+        __syncthreads();
+        if (threadIdx.x >= 32) return;
+        const int q = lane >> 2, i0 = (lane & 3) * 8;
+        double v = 0.0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v += (double)sh[q][i0 + i];
+        v += shfl_xor(v, 1);
+        v += shfl_xor(v, 2);
+        if ((lane & 3) == 0 && shc[q] >= 0) part_loss[shc[q]] = v;
+    } else {
+        const double ls = warp_sum((double)lsum);
+        if (lane == 0) part_loss[c] = ls;
+    }
 }
 
 // Sums of S <= 8 values over the warp, every lane receiving all of them, with
@@ -285,21 +358,35 @@ __device__ __forceinline__ void warp_sum_vec(double (&g)[S])
         g[i] = __shfl_sync(0xffffffffu, v[0], ((i >> 2) & 1) | (((i >> 1) & 1) << 1) | ((i & 1) << 2));
 }
 
+// Two warp sums, every lane receiving both, in 5 additions instead of 10: the
+// first step splits the values over the half warps.  The pairs and their order
+// are those of warp_sum.
+__device__ __forceinline__ void warp_sum_two(double a, double b, double &sa, double &sb)
+{
+    const bool up = (threadIdx.x & 16) != 0;
+    double v = (up ? b : a) + shfl_xor(up ? a : b, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v += shfl_xor(v, o);
+    sa = __shfl_sync(0xffffffffu, v, 0);
+    sb = __shfl_sync(0xffffffffu, v, 16);
+}
+
 // A whole half-step of segments that fit in one chunk, a warp per segment:
 // gradient pass, prox, loss pass of the candidate, decision.  The candidate's
 // coordinates stay in the lanes that hold the gradient's (every lane group
 // has the whole row), so nothing goes through memory between the steps: one
 // launch of the four and no partials.  On the 200 x 100, k = 5 FP64 table,
-// whose half-steps are launch- and latency-bound, 18 and 23 us (masked tiles:
-// 200 and 272 us); 10.6 -> 10.3 ms for the 1,000,000 rows (200 entries, k = 64)
-// of the completion table.
-template <class T, int K, bool XSTEP, bool VEC>
+// whose half-steps are launch- and latency-bound, 15 and 20 us (masked tiles:
+// 200 and 272 us); the 1,000,000 rows (200 entries, k = 64) of the completion
+// table, bound by the gathers from L2: 10.6 ms in four launches, 10.3 in one,
+// 7.9 with the indices loaded one group ahead.
+template <class T, int K, bool XSTEP, int VEC>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
 seg_kernel(int64_t nseg, const int32_t *__restrict__ ptr, const int32_t *__restrict__ idx,
            const T *__restrict__ val, T *__restrict__ F, const T *__restrict__ W, int k,
            const LossOf<T> *__restrict__ loss, T *__restrict__ alpha, int rkind, T rw,
            double *__restrict__ kept_obj, double *__restrict__ kept_reg, int32_t *__restrict__ accepted,
-           const T *__restrict__ lsc)
+           const T *__restrict__ lsc, bool uni)
 {
     using LN = Lanes<K>;
     constexpr int G = LN::G, S = LN::S, PER = LN::PER;
@@ -316,18 +403,28 @@ seg_kernel(int64_t nseg, const int32_t *__restrict__ ptr, const int32_t *__restr
     for (int q = 0; q < S; ++q) g[q] = T(0);
     LossOf<T> sp;
     T wsc = T(1);
-    if constexpr (!XSTEP) {
+    if constexpr (XSTEP) {
+        sp = loss[0];  // of every column, when uni
+    } else {
         sp = loss[s];
         if (lsc) wsc = __ldg(lsc + s);
     }
-    // loss (and derivative) of entry q at f, its row in w
+    // loss (and derivative) of entry q at f, its row in w; the index and value
+    // of the next group's entry are on their way while the row waits
+    int jn = 0;
+    T an = T(0);
+    auto ahead = [&](int q) {
+        if (q < e) {
+            jn = __ldg(idx + q);
+            an = __ldg(val + q);
+        }
+    };
     auto entry = [&](int q, const T (&x)[S], T (&w)[S], T &L) -> T {
         const bool in = q < e;
-        int j = 0;
-        T a = T(0);
+        const int j = jn;
+        const T a = an;
+        ahead(q + PER);
         if (in) {
-            j = __ldg(idx + q);
-            a = __ldg(val + q);
             load_lane<T, S, G, VW, VEC>(w, W + (int64_t)j * k, gl, k);
         } else {
 #pragma unroll
@@ -342,7 +439,7 @@ seg_kernel(int64_t nseg, const int32_t *__restrict__ ptr, const int32_t *__restr
         L = T(0);
         if (in) {
             if constexpr (XSTEP) {
-                sp = loss[j];
+                if (!uni) sp = loss[j];
                 if (lsc) wsc = __ldg(lsc + j);
             }
             d = loss_deriv<T>(sp, u, a, L);
@@ -354,6 +451,7 @@ seg_kernel(int64_t nseg, const int32_t *__restrict__ ptr, const int32_t *__restr
         return d;
     };
     T lsum = T(0);
+    ahead(b + grp);
     for (int q = b; q < e; q += PER) {
         T w[S], L;
         const T d = entry(q + grp, f, w, L);
@@ -370,7 +468,6 @@ seg_kernel(int64_t nseg, const int32_t *__restrict__ ptr, const int32_t *__restr
             for (int o = G; o < 32; o <<= 1) g[c] += shfl_xor(g[c], o);
         }
     }
-    const double fo_loss = warp_sum((double)lsum);
     // the candidate, in the lanes' own coordinates
     T ro = T(0), rn = T(0);
 #pragma unroll
@@ -392,25 +489,26 @@ seg_kernel(int64_t nseg, const int32_t *__restrict__ ptr, const int32_t *__restr
     // losses of the candidate, the next group of entries on its way while the
     // current one is evaluated (as in the loss passes of pass_kernel)
     T lsum2 = T(0);
-    T an = T(0), wn[S], wscn = wsc;
+    T av = T(0), wn[S], wscn = wsc;
     LossOf<T> spn = sp;
     auto fetch = [&](int q) {
         if (q < e) {
-            const int j = __ldg(idx + q);
-            an = __ldg(val + q);
-            load_lane<T, S, G, VW, VEC>(wn, W + (int64_t)j * k, gl, k);
+            av = an;
+            load_lane<T, S, G, VW, VEC>(wn, W + (int64_t)jn * k, gl, k);
             if constexpr (XSTEP) {
-                spn = loss[j];
-                if (lsc) wscn = __ldg(lsc + j);
+                if (!uni) spn = loss[jn];
+                if (lsc) wscn = __ldg(lsc + jn);
             }
+            ahead(q + PER);
         } else {
 #pragma unroll
             for (int c = 0; c < S; ++c) wn[c] = T(0);
         }
     };
+    ahead(b + grp);
     fetch(b + grp);
     for (int q = b; q < e; q += PER) {
-        const T a = an;
+        const T a = av;
         T u = T(0);
 #pragma unroll
         for (int c = 0; c < S; ++c) u = fma(f[c], wn[c], u);
@@ -426,7 +524,10 @@ seg_kernel(int64_t nseg, const int32_t *__restrict__ ptr, const int32_t *__restr
             if (gl == 0) lsum2 += L;
         }
     }
-    const double fn = warp_sum((double)lsum2) + rn, fo = fo_loss + ro;
+    double fo, fn;
+    warp_sum_two((double)lsum, (double)lsum2, fo, fn);
+    fo += ro;
+    fn += rn;
     const bool acc = fn <= fo;
     if (acc && grp == 0) {
 #pragma unroll
@@ -924,36 +1025,38 @@ __global__ void reset_alpha_kernel(const int32_t *__restrict__ ptr, int64_t nseg
 template <class T, int K, bool XSTEP, bool GRAD, class WT>
 cudaError_t launch_pass(const Orient &o, const T *F, const WT *W, int k, const LossOf<T> *loss,
                         T *part_grad, double *part_loss, cudaStream_t st, const int32_t *sel, int want,
-                        const T *lsc)
+                        const T *lsc, bool uni)
 {
     if (o.nchunks == 0) return cudaSuccess;
     // the BF16 copy is read 8 values at a time, so its vector path needs k % 8 == 0
-    constexpr int kVecMult = std::is_same<WT, __nv_bfloat16>::value ? 8 : 1;
-    const bool vec = (k == K) && (Lanes<K>::S % kVecMult == 0) &&
-                     ((reinterpret_cast<uintptr_t>(F) | reinterpret_cast<uintptr_t>(W)) % 16 == 0);
+    constexpr bool kBf = std::is_same<WT, __nv_bfloat16>::value;
+    constexpr int kVecMult = kBf ? 8 : 1;
+    const uintptr_t at = reinterpret_cast<uintptr_t>(F) | reinterpret_cast<uintptr_t>(W);
+    const bool vec = (k == K) && (Lanes<K>::S % kVecMult == 0) && at % 16 == 0;
     const unsigned nb = blocks_for(o.nchunks, kWarpsPerBlock);
-    if constexpr (std::is_same<WT, __nv_bfloat16>::value && Lanes<K>::S % 8 != 0) {
-        pass_kernel<T, K, XSTEP, false, GRAD, WT><<<nb, kWarpsPerBlock * 32, 0, st>>>(
-            o.nchunks, o.chunks, o.order, o.idx, (const T *)o.val, F, W, k, loss, part_grad, part_loss, sel, want, lsc);
-    } else {
-        if (vec)
-            pass_kernel<T, K, XSTEP, true, GRAD, WT><<<nb, kWarpsPerBlock * 32, 0, st>>>(
-                o.nchunks, o.chunks, o.order, o.idx, (const T *)o.val, F, W, k, loss, part_grad, part_loss, sel, want, lsc);
-        else
-            pass_kernel<T, K, XSTEP, false, GRAD, WT><<<nb, kWarpsPerBlock * 32, 0, st>>>(
-                o.nchunks, o.chunks, o.order, o.idx, (const T *)o.val, F, W, k, loss, part_grad, part_loss, sel, want, lsc);
+    auto go = [&](auto kern) {
+        kern<<<nb, kWarpsPerBlock * 32, 0, st>>>(o.nchunks, o.chunks, o.order, o.idx, (const T *)o.val, F, W, k, loss,
+                                                 part_grad, part_loss, sel, want, lsc, uni);
+        return cudaGetLastError();
+    };
+    if constexpr (!kBf || Lanes<K>::S % 8 == 0) {
+        if (vec) return go(pass_kernel<T, K, XSTEP, kUnits, GRAD, WT>);
     }
-    return cudaGetLastError();
+    if constexpr (pairs_ok<WT, K>) {
+        if (k % 2 == 0 && at % 8 == 0) return go(pass_kernel<T, K, XSTEP, kPairs, GRAD, WT>);
+    }
+    return go(pass_kernel<T, K, XSTEP, kScalar, GRAD, WT>);
 }
 
 // Dispatch a runtime k to the smallest padded width K >= k.
 template <class T, bool XSTEP, bool GRAD, class WT = T>
 cudaError_t dispatch_pass(const Orient &o, const T *F, const WT *W, int k, const LossOf<T> *loss,
                           T *part_grad, double *part_loss, cudaStream_t st, const int32_t *sel = nullptr,
-                          int want = 0, const T *lsc = nullptr)
+                          int want = 0, const T *lsc = nullptr, bool uni = false)
 {
 #define GLRM_PASS_CASE(KK) \
-    if (k <= KK) return launch_pass<T, KK, XSTEP, GRAD, WT>(o, F, W, k, loss, part_grad, part_loss, st, sel, want, lsc);
+    if (k <= KK)           \
+        return launch_pass<T, KK, XSTEP, GRAD, WT>(o, F, W, k, loss, part_grad, part_loss, st, sel, want, lsc, uni);
     GLRM_PASS_CASE(4)
     GLRM_PASS_CASE(8)
     GLRM_PASS_CASE(12)
@@ -973,7 +1076,7 @@ cudaError_t run_pass(glrm_s *h, const T *F, const T *W, T *part_grad, double *pa
                      int want = 0, const T *lsc = nullptr)
 {
     return dispatch_pass<T, XSTEP, GRAD>(XSTEP ? h->csr : h->csc, F, W, h->k, loss_of<T>(h), part_grad, part_loss,
-                                         h->stream, sel, want, lsc);
+                                         h->stream, sel, want, lsc, h->loss_uniform);
 }
 
 // The BF16 form's gradient passes: the other factor's rows from a BF16 copy.
@@ -983,14 +1086,16 @@ cudaError_t run_pass_bf16(glrm_s *h, const float *F, const __nv_bfloat16 *W, flo
 {
     if (staged_bf16_ok(h->k, W)) return staged_pass_bf16(h, XSTEP, F, W, part_grad, part_loss, sel, want);
     return dispatch_pass<float, XSTEP, true, __nv_bfloat16>(XSTEP ? h->csr : h->csc, F, W, h->k, h->loss_f, part_grad,
-                                                            part_loss, h->stream, sel, want);
+                                                            part_loss, h->stream, sel, want, nullptr,
+                                                            h->loss_uniform);
 }
 
 template <class T, int K, bool XSTEP>
 cudaError_t launch_seg(glrm_s *h, const Orient &o, T *F, const T *W, T *alpha, int rk, T rw)
 {
     Scratch &s = h->s;
-    const bool vec = h->k == K && (reinterpret_cast<uintptr_t>(F) | reinterpret_cast<uintptr_t>(W)) % 16 == 0;
+    const uintptr_t at = reinterpret_cast<uintptr_t>(F) | reinterpret_cast<uintptr_t>(W);
+    const bool vec = h->k == K && at % 16 == 0;
     // few segments: fewer warps per block, so that they spread over the SMs
     int warps = kWarpsPerBlock;
     while (warps > 1 && o.nseg < 152LL * warps) warps /= 2;
@@ -999,16 +1104,17 @@ cudaError_t launch_seg(glrm_s *h, const Orient &o, T *F, const T *W, T *alpha, i
         kern<<<nb, warps * 32, 0, h->stream>>>(
             o.nseg, o.ptr, o.idx, (const T *)o.val, F, W, h->k, loss_of<T>(h), alpha, rk, rw,
             XSTEP ? s.kept_obj_x : s.kept_obj_y, XSTEP ? s.kept_reg_x : s.kept_reg_y, XSTEP ? s.acc_x : s.acc_y,
-            (const T *)h->lscale);
+            (const T *)h->lscale, h->loss_uniform);
+        h->launches += 1;
+        return cudaGetLastError();
     };
     if constexpr (K % 4 == 0) {
-        if (vec) go(seg_kernel<T, K, XSTEP, true>);
-        else go(seg_kernel<T, K, XSTEP, false>);
-    } else {
-        go(seg_kernel<T, K, XSTEP, false>);
+        if (vec) return go(seg_kernel<T, K, XSTEP, kUnits>);
     }
-    h->launches += 1;
-    return cudaGetLastError();
+    if constexpr (pairs_ok<T, K>) {
+        if (h->k % 2 == 0 && at % 8 == 0) return go(seg_kernel<T, K, XSTEP, kPairs>);
+    }
+    return go(seg_kernel<T, K, XSTEP, kScalar>);
 }
 
 template <class T, bool XSTEP>
