@@ -508,10 +508,13 @@ int glrm_set_state(glrm_t h, const void *buf_host, size_t len);
  *   GLRM_PATH_DENSE    (both half-steps) the table stored densely with NaN at
  *                      the missing cells and swept by the tensor-core form of
  *                      glrm_set_dense; FP32 and BF16 models with k <= 64
- * GLRM_PATH_AUTO picks dense for FP32 and BF16 models with k <= 64 when at least 40% of
- * the cells are observed (and the dense copy takes at most half the free
- * device memory); otherwise masked when a tile's pairs average >= 8 observed
- * lanes (chunked when that gives fewer than 48 units of work), else fused when the other factor fits, else blocked when a
+ * GLRM_PATH_AUTO picks dense for FP32 and BF16 models with k <= 64 when at least
+ * 40% of the cells are observed (and the dense copy takes at most half the free
+ * device memory).  Otherwise an FP32 half-step whose segments average >= 4096
+ * entries is chunked; any is masked when a tile's pairs average >= 8 observed
+ * lanes (chunked when that gives fewer than 48 units of work); the other FP32
+ * ones are chunked when their segments average >= 8 entries (rows of an odd
+ * k > 16 excepted); else fused when the other factor fits, else blocked when a
  * (panel, segment) run holds >= 64 entries on average, else chunked.  The
  * staged paths need k <= 32.  glrm_set_path(h, xstep_path, ystep_path) may be
  * called before or after glrm_set_observed; an infeasible request returns

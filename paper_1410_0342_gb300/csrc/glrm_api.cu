@@ -121,10 +121,40 @@ int tiled_width(int k)
     return 0;
 }
 
+// Density from which an FP32 observed set is stored densely (NaN marking the
+// missing cells) and swept by the tensor-core form.  Below it the dense sweeps
+// are still the faster ones on large tables (50,021 x 701, k = 18, 25%: 414
+// against 850 us), but the split products' factors are further from the FP64
+// sweep's there than the sparse paths' (5.1e-7 against 5.2e-8 relative).
+constexpr double kDenseAutoDensity = 0.4;
+
 // Pick fused / blocked / chunked for one orientation: fused when the whole
 // other factor (plus, for the X-step, its loss table) fits in one CTA's shared
 // memory; blocked when panels of it do and a (panel, segment) run holds 64
-// entries or more on average; chunked otherwise.
+// entries or more on average; chunked otherwise, and where chunked_first says
+// so.
+
+// FP32 tables below the dense form's density: where the chunked half-steps
+// beat the staged ones (sweep us, staged -> chunked in that orientation).
+// Before masked tiles: segments of 4,096 entries or more, four warps each
+// (columns of 20,000 x 300 k = 20 at 33%: 331 -> 211, 100,000 x 1,000 k = 20:
+// 1741 -> 1548, 400,000 x 200 k = 8: 1255 -> 664; rows stay masked, of 400,000
+// 1255 against 1409).  Otherwise before the fused and blocked forms: segments
+// of 8 entries or more (50,021 x 701, 25%, k = 18: rows 768 -> 680, columns
+// 768 -> 649; 600,000 x 300, 10%, k = 32: 6593 -> 4760 and 5534; 60,000 x
+// 3,000 with rows of 15, k = 8: 224 -> 96; blocked rows of 300 x 5,000, 20%:
+// 203 -> 85), but not rows of a larger odd rank, which load coordinate by
+// coordinate (k = 19: 780 -> 830, k = 17: 739 -> 731).  Shorter segments keep
+// the fused form (rows of 6 would also gain, 200 -> 90).  FP64 half-steps are
+// bound by their arithmetic on either path (fused rows 3992, chunked 4114).
+bool chunked_first(const glrm_s *h, const Orient &o, bool xstep, bool before_masked)
+{
+    const double len = (double)h->nnz / (double)o.nseg, cells = (double)h->m * (double)h->n;
+    if (h->prec != GLRM_FP32 || (double)h->nnz >= kDenseAutoDensity * cells) return false;
+    if (before_masked) return len >= 4096.0;
+    return len >= 8.0 && (!xstep || h->k % 2 == 0 || h->k <= 16);
+}
+
 // Units (warps) below which the automatic choice prefers the chunked form to
 // masked tiles: on the 200 x 100, k = 5 FP64 table (7 and 4 units) the masked
 // half-steps take 200 and 272 us, the chunked ones 18 and 23 us.
@@ -267,6 +297,7 @@ int choose_mode(glrm_s *h, Orient &o, bool xstep, int force)
         if (force == GLRM_PATH_AUTO) return GLRM_OK;
         return fail(h, GLRM_ERR_ARG, "the staged paths need 1 <= k <= 32 and a non-empty Omega");
     }
+    if (force == GLRM_PATH_AUTO && chunked_first(h, o, xstep, true)) return GLRM_OK;
     const size_t es = elem_size(h->prec);
     const int64_t nother = xstep ? h->n : h->m;
     const size_t per_row = (size_t)K * es + (xstep ? sizeof(LossSpec) : 0);
@@ -276,6 +307,7 @@ int choose_mode(glrm_s *h, Orient &o, bool xstep, int force)
         int rc = plan_masked(h, o, xstep, force, K, sms, budget, small);
         if (rc != GLRM_OK || o.mode == kModeMasked || force != GLRM_PATH_AUTO || small) return rc;
     }
+    if (force == GLRM_PATH_AUTO && chunked_first(h, o, xstep, false)) return GLRM_OK;
     // per warp: two staging buffers of `cap` (index, value) pairs
     const size_t per_cap = (size_t)kStreamWarps * 2 * (sizeof(int32_t) + es);
     const size_t panel_all = ((((size_t)nother * K * es) + 15) & ~(size_t)15) +
@@ -453,13 +485,6 @@ const char *flag_message(int f)
     if (f & 64) return "a value outside its column loss's domain (Boolean: -1 or +1; ordinal: integer in 1..d)";
     return "invalid observed set";
 }
-
-// Density from which an FP32 observed set is stored densely (NaN marking the
-// missing cells) and swept by the tensor-core form.  Below it the dense sweeps
-// are still the faster ones on large tables (50,021 x 701, k = 18, 25%: 414
-// against 850 us), but the split products' factors are further from the FP64
-// sweep's there than the sparse paths' (5.1e-7 against 5.2e-8 relative).
-constexpr double kDenseAutoDensity = 0.4;
 
 // Whether the observed set goes to the dense form: 1 yes, 0 no, else a
 // GLRM error code (a dense request the model cannot take).
