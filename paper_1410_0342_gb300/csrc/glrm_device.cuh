@@ -355,6 +355,19 @@ __device__ __forceinline__ T warp_sum(T v)
     return v;
 }
 
+// Two warp sums, every lane receiving both, in 5 additions instead of 10: the
+// first step splits the values over the half warps.  The pairs and their order
+// are those of warp_sum.
+__device__ __forceinline__ void warp_sum_two(double a, double b, double &sa, double &sb)
+{
+    const bool up = (threadIdx.x & 16) != 0;
+    double v = (up ? b : a) + shfl_xor(up ? a : b, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v += shfl_xor(v, o);
+    sa = __shfl_sync(0xffffffffu, v, 0);
+    sb = __shfl_sync(0xffffffffu, v, 16);
+}
+
 // Load coordinates c0 .. c0+S-1 of a factor row (row-major, k values).
 // VEC: the caller guarantees k == the padded width, so the slice is in range,
 // and 16-byte alignment, so the slice loads as float4 / double2 vectors.

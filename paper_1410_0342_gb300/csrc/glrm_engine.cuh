@@ -358,19 +358,6 @@ __device__ __forceinline__ void warp_sum_vec(double (&g)[S])
         g[i] = __shfl_sync(0xffffffffu, v[0], ((i >> 2) & 1) | (((i >> 1) & 1) << 1) | ((i & 1) << 2));
 }
 
-// Two warp sums, every lane receiving both, in 5 additions instead of 10: the
-// first step splits the values over the half warps.  The pairs and their order
-// are those of warp_sum.
-__device__ __forceinline__ void warp_sum_two(double a, double b, double &sa, double &sb)
-{
-    const bool up = (threadIdx.x & 16) != 0;
-    double v = (up ? b : a) + shfl_xor(up ? a : b, 16);
-#pragma unroll
-    for (int o = 8; o > 0; o >>= 1) v += shfl_xor(v, o);
-    sa = __shfl_sync(0xffffffffu, v, 0);
-    sb = __shfl_sync(0xffffffffu, v, 16);
-}
-
 // A whole half-step of segments that fit in one chunk, a warp per segment:
 // gradient pass, prox, loss pass of the candidate, decision.  The candidate's
 // coordinates stay in the lanes that hold the gradient's (every lane group
