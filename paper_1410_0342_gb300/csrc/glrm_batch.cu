@@ -123,13 +123,16 @@ struct BVec {
     float v[K];
 };
 
+// A factor row.  Plain loads: the launch itself writes the factors (an item
+// reads the rows that the items it waited for have stored), and the read-only
+// path (__ldg) is only for memory that nothing writes while the kernel runs.
 template <int K>
-__device__ __forceinline__ void bload(float (&v)[K], const float *__restrict__ row)
+__device__ __forceinline__ void bload(float (&v)[K], const float *row)
 {
     const float4 *p = reinterpret_cast<const float4 *>(row);
 #pragma unroll
     for (int q = 0; q < K / 4; ++q) {
-        const float4 t = __ldg(p + q);
+        const float4 t = p[q];
         v[4 * q] = t.x;
         v[4 * q + 1] = t.y;
         v[4 * q + 2] = t.z;
