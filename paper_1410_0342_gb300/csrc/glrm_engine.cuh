@@ -51,15 +51,25 @@ __device__ __forceinline__ int slot_coord(int s, int gl)
     return VEC == kUnits ? VW * ((s / VW) * G + gl) + s % VW : gl * S + s;
 }
 
-// A row's slots for lane gl in the layout above (T values, units of VW).
-template <class T, int S, int G, int VW, int VEC>
-__device__ __forceinline__ void load_lane(T (&v)[S], const T *__restrict__ row, int gl, int k)
+// One value (or vector) of a factor: through the read-only path, or by a plain
+// load where the launch itself writes that factor.
+template <bool RO, class V>
+__device__ __forceinline__ V load_factor(const V *p)
+{
+    if constexpr (RO) return __ldg(p);
+    else return *p;
+}
+
+// A row's slots for lane gl in the layout above (T values, units of VW).  RO:
+// nothing writes the factor during the launch.
+template <class T, int S, int G, int VW, int VEC, bool RO = true>
+__device__ __forceinline__ void load_lane(T (&v)[S], const T *row, int gl, int k)
 {
     if constexpr (VEC == kPairs) {
         static_assert(G == 1 && S % 2 == 0 && sizeof(T) == 4, "pairs are of whole FP32 rows");
 #pragma unroll
         for (int q = 0; q < S / 2; ++q) {
-            const float2 t = 2 * q < k ? __ldg(reinterpret_cast<const float2 *>(row) + q) : make_float2(0.f, 0.f);
+            const float2 t = 2 * q < k ? load_factor<RO>(reinterpret_cast<const float2 *>(row) + q) : make_float2(0.f, 0.f);
             v[2 * q] = t.x;
             v[2 * q + 1] = t.y;
         }
@@ -72,13 +82,13 @@ __device__ __forceinline__ void load_lane(T (&v)[S], const T *__restrict__ row, 
             for (int h = 0; h < VW / VT; ++h) {
                 const T *src = row + VW * (q * G + gl) + VT * h;
                 if constexpr (sizeof(T) == 4) {
-                    const float4 t = __ldg(reinterpret_cast<const float4 *>(src));
+                    const float4 t = load_factor<RO>(reinterpret_cast<const float4 *>(src));
                     v[q * VW + VT * h + 0] = t.x;
                     v[q * VW + VT * h + 1] = t.y;
                     v[q * VW + VT * h + 2] = t.z;
                     v[q * VW + VT * h + 3] = t.w;
                 } else {
-                    const double2 t = __ldg(reinterpret_cast<const double2 *>(src));
+                    const double2 t = load_factor<RO>(reinterpret_cast<const double2 *>(src));
                     v[q * VW + VT * h + 0] = t.x;
                     v[q * VW + VT * h + 1] = t.y;
                 }
@@ -86,7 +96,7 @@ __device__ __forceinline__ void load_lane(T (&v)[S], const T *__restrict__ row, 
         }
     } else {
 #pragma unroll
-        for (int s = 0; s < S; ++s) v[s] = (gl * S + s < k) ? __ldg(row + gl * S + s) : T(0);
+        for (int s = 0; s < S; ++s) v[s] = (gl * S + s < k) ? load_factor<RO>(row + gl * S + s) : T(0);
     }
 }
 
@@ -385,7 +395,7 @@ seg_kernel(int64_t nseg, const int32_t *__restrict__ ptr, const int32_t *__restr
     const int b = ptr[s], e = ptr[s + 1];
     const T al = alpha[s];
     T f[S], g[S];
-    load_lane<T, S, G, VW, VEC>(f, F + s * k, gl, k);
+    load_lane<T, S, G, VW, VEC, false>(f, F + s * k, gl, k);  // (stored again after the decision)
 #pragma unroll
     for (int q = 0; q < S; ++q) g[q] = T(0);
     LossOf<T> sp;
