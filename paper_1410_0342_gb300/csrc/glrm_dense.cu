@@ -53,10 +53,11 @@ constexpr int kDnRows = 128;     // own rows per CTA (UMMA M)
 constexpr int kDnWarps = 16;     // evaluating warp w: TMEM lanes 32 (w % 4) .. + 31, chunk columns 16 (w / 4) .. + 15
 constexpr int kDnThreads = (kDnWarps + 3) * 32;  // + the GEMM1 warp, the copy warp, the GEMM2 warp
 // TMEM columns: U at [0, 64) and [64, 128), two buffers of R (hi, mid, lo; 32
-// columns each) at [128, 224) and [224, 320), G at [320, 320 + KP), the own
-// rows (hi, mid, lo; KP / 2 columns each) from 384
+// columns each) at [128, 224) and [224, 320), G from 320 (two accumulators of
+// up to 48 columns or one of 64), the own rows (hi, mid, lo; KP / 2 columns
+// each) from 416
 constexpr int kDnTmem = 512;
-constexpr int kDnColR = 128, kDnColG = 320, kDnColOwn = 384;
+constexpr int kDnColR = 128, kDnColG = 320, kDnColOwn = 416;
 constexpr int kDnMaxStages = 4;
 
 // Column loss with its parameters in FP32 (kind as int bits, Huber
@@ -471,6 +472,15 @@ dense_pass_kernel(const DenseArgs p, const __grid_constant__ CUtensorMap amap)
     const int64_t qb = item.q0;
     const int nq = item.nq;
     const int nA = p.nA;
+    // GEMM2's width in coordinates, and whether its hi . hi products have an
+    // accumulator of their own.  An MMA rounds the running sum it adds to, so
+    // with all six products in one accumulator the five small ones of every
+    // chunk cost as much rounding as the large one: 24 roundings a chunk instead
+    // of 4 (error of Yt after a sweep of the 100,000 x 1,000 mixed table,
+    // k = 20: 1.02e-6 against 9.7e-8; time 688 against 691 us).  Ranks over 48 leave no
+    // columns for a second one.
+    const int gw = KP <= 32 ? KP : (p.k <= 48 ? 48 : 64);
+    const bool two = !B16 && gw <= 48;
     const bool producer = warp >= kDnWarps;  // kDnWarps: GEMM1, kDnWarps + 1: copies, kDnWarps + 2: GEMM2
     // this thread's own row (X-step) or column (Y-step: quarter q of the tile
     // is the 32-column block blocks[4 tile + q]), and its partial slot
@@ -668,18 +678,18 @@ dense_pass_kernel(const DenseArgs p, const __grid_constant__ CUtensorMap amap)
                 // them on a table of Boolean and ordinal columns)
                 uint32_t wh[4];
                 *reinterpret_cast<uint4 *>(wh) = *reinterpret_cast<const uint4 *>(whole_s[c & 3]);
-                constexpr uint32_t idesc = umma_idesc_bf16(kDnRows, KP);
+                const uint32_t idesc = umma_idesc_bf16(kDnRows, gw);
                 constexpr int P0 = B16 ? 5 : 0;  // the BF16 form: hi . hi only
 #pragma unroll
                 for (int pr = P0; pr < 6; ++pr)
 #pragma unroll
-                    for (int ks = 0; ks < kDnNT / 16; ++ks)
-                        if (pr == P0 && ks == 0) {  // the first MMA of chunk 0 sets G
-                            umma_bf16_ta(taddr + kDnColG, r0 + pa[pr] * 32, d0 + (pb[pr] * SM::pt >> 4), idesc, c > 0);
-                        } else if (pa[pr] == 0 || wh[ks] != 0x01010101u) {
-                            umma_bf16_ta(taddr + kDnColG, r0 + pa[pr] * 32 + ks * 8,
-                                         d0 + ((pb[pr] * SM::pt + ks * 32) >> 4), idesc, true);
-                        }
+                    for (int ks = 0; ks < kDnNT / 16; ++ks) {
+                        // an accumulator's first MMA of chunk 0 sets it
+                        const bool first = ks == 0 && (pr == P0 || (pr == 5 && two));
+                        if ((pr == P0 && ks == 0) || pa[pr] == 0 || wh[ks] != 0x01010101u)
+                            umma_bf16_ta(taddr + kDnColG + (two && pr < 5 ? gw : 0), r0 + pa[pr] * 32 + ks * 8,
+                                         d0 + ((pb[pr] * SM::pt + ks * 32) >> 4), idesc, c > 0 || !first);
+                    }
                 umma_commit(&barG2[c & 3]);
                 ++g2_issued;
             }
@@ -886,8 +896,20 @@ dense_pass_kernel(const DenseArgs p, const __grid_constant__ CUtensorMap amap)
             float *g = p.part_grad + slot * p.k;
 #pragma unroll
             for (int bb = 0; bb < KP / 16; ++bb) {
+                if (16 * bb >= gw) break;
                 float v[16];
-                tmem_ld16(taddr + lane_base + (uint32_t)(kDnColG + 16 * bb), v);
+                if (two) {
+                    uint32_t hi[16], lo[16];
+                    float low[16];
+                    tmem_ld16_start(taddr + lane_base + (uint32_t)(kDnColG + 16 * bb), hi);
+                    tmem_ld16_start(taddr + lane_base + (uint32_t)(kDnColG + gw + 16 * bb), lo);
+                    tmem_ld16_wait(hi, v);
+                    tmem_ld16_wait(lo, low);
+#pragma unroll
+                    for (int w = 0; w < 16; ++w) v[w] += low[w];
+                } else {
+                    tmem_ld16(taddr + lane_base + (uint32_t)(kDnColG + 16 * bb), v);
+                }
                 if (own_ok) {
 #pragma unroll
                     for (int w = 0; w < 16; ++w)
