@@ -463,7 +463,8 @@ __device__ __forceinline__ int load_acquire(const int32_t *p)
 }
 
 // Whole warp: wait until *ctr >= target (lane 0 polls, at most `limit`
-// times, and gives up at once when the error flag is up).  True when the
+// times, and gives up at once when another wait has run out; a failed
+// factorisation, the flag's other bit, leaves the counters right).  True when the
 // condition holds; the writes counted by *ctr are then visible to every lane.
 __device__ bool warp_wait_count(const int32_t *ctr, int target, long long limit, int *err)
 {
@@ -472,7 +473,7 @@ __device__ bool warp_wait_count(const int32_t *ctr, int target, long long limit,
     if (lane == 0) {
         long long it = 0;
         while (load_acquire(ctr) < target) {
-            if (it++ >= limit || *(volatile int *)err) {
+            if (it++ >= limit || (*(volatile int *)err & kErrWait)) {
                 ok = 0;
                 break;
             }
