@@ -721,10 +721,12 @@ void build_items(const glrm_batch_s *b, bool xstep, const int32_t *tiles, const 
 
 // Tile sizes before autotuning, per bucket: 512 entries an item (the size
 // class's typical segment: 32, 128, 512, 2048 entries), at least a lane group
-// for ALS, halved while the batch has fewer than 8 items for each of about
-// 4,800 resident warps in a half-step.
+// for ALS, halved while a half-step of the batch has fewer than 8 items for each
+// resident warp (2,432: two CTAs of eight warps on each of 152 SMs; with twice
+// that many assumed, 50 instances took 1.38 instead of 1.32 ms a sweep).
 void default_tiles(glrm_batch_s *b)
 {
+    const int64_t warps = (int64_t)b->qgrid * kBWarps;
     int64_t segs_x = 0, segs_y = 0;
     for (const BInst &I : b->inst_host) {
         segs_x += I.m;
@@ -736,7 +738,7 @@ void default_tiles(glrm_batch_s *b)
         for (int half = 0; half < 2; ++half) {
             const int64_t segs = half == 0 ? segs_x : segs_y;
             int t = std::max(1, 512 / lens[cls]);
-            while (t > 1 && segs / t < 8 * 4800) t /= 2;
+            while (t > 1 && segs / t < 8 * warps) t /= 2;
             if (method == GLRM_BATCH_ALS) t = std::max(t, 32 / kc);
             (half == 0 ? b->tile_x : b->tile_y)[q] = t;
         }
@@ -911,12 +913,6 @@ int glrm_batch_create(int32_t count, const glrm_batch_instance *ih, const int32_
     b->cols = cb;
     b->xlen = xo;
     b->ylen = yo;
-    // work items before any autotuning: an ALS item fills its lane groups
-    // (32 / k rows), and an item holds about 512 entries (an item per row
-    // leaves short rows paying for the queue: one atomic, one fence and the
-    // counter waits each), as long as the batch still gives several items to
-    // every warp
-    default_tiles(b);
     BCK(cudaGetDevice(&b->device));
     int sms = 0;
     BCK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device));
@@ -926,6 +922,12 @@ int glrm_batch_create(int32_t count, const glrm_batch_instance *ih, const int32_
     BCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_queue_kernel, kBWarps * 32,
                                                       kBWarps * kAlsWarpBytes));
     b->qgrid = sms * std::max(per_sm, 1);
+    // work items before any autotuning: an ALS item fills its lane groups
+    // (32 / k rows), and an item holds about 512 entries (an item per row
+    // leaves short rows paying for the queue: one atomic, one fence and the
+    // counter waits each), as long as the batch still gives several items to
+    // every warp
+    default_tiles(b);
     BCK(cudaStreamCreateWithFlags(&b->capture, cudaStreamNonBlocking));
     cudaStream_t st = b->stream;
     const size_t nz = (size_t)std::max<int64_t>(e, 1);
