@@ -211,13 +211,13 @@ __device__ __forceinline__ void dn_block_loop(const float (&u)[16], const float 
 
 // The losses and derivatives of the scalar functions the sparse paths use,
 // for kinds without a packed form.
-template <int KIND>
+template <int KIND, bool MISS>
 __device__ __forceinline__ void dn_block_plain(const float (&u)[16], const float (&a)[16], float prm, float lev,
                                                float (&rr)[16], float &lsum)
 {
 #pragma unroll
     for (int w = 0; w < 16; ++w) {
-        const bool v = a[w] == a[w];
+        const bool v = !MISS || a[w] == a[w];
         float L;
         const float d = loss_deriv_k<KIND, float>(u[w], a[w], prm, lev, L);
         lsum += v ? L : 0.f;
@@ -361,7 +361,7 @@ __device__ __forceinline__ void dn_block(const float (&u)[16], const float (&a)[
             upk2(q, rr[w], rr[w + 1]);
         }
     } else {
-        dn_block_plain<KIND>(u, a, prm, lev, rr, lsum);
+        dn_block_plain<KIND, MISS>(u, a, prm, lev, rr, lsum);
     }
     float l0, l1;
     upk2(acc, l0, l1);

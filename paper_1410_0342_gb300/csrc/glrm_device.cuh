@@ -368,37 +368,4 @@ __device__ __forceinline__ void warp_sum_two(double a, double b, double &sa, dou
     sb = __shfl_sync(0xffffffffu, v, 16);
 }
 
-// Load coordinates c0 .. c0+S-1 of a factor row (row-major, k values).
-// VEC: the caller guarantees k == the padded width, so the slice is in range,
-// and 16-byte alignment, so the slice loads as float4 / double2 vectors.
-// Otherwise coordinates at or beyond k read as 0.
-template <class T, int S, bool VEC>
-__device__ __forceinline__ void load_slice(T (&v)[S], const T *__restrict__ row, int c0, int k)
-{
-    if constexpr (VEC && sizeof(T) == 4) {
-        static_assert(S % 4 == 0, "float slice must be a multiple of 4");
-        const float4 *p = reinterpret_cast<const float4 *>(row + c0);
-#pragma unroll
-        for (int q = 0; q < S / 4; ++q) {
-            float4 t = __ldg(p + q);
-            v[4 * q + 0] = t.x;
-            v[4 * q + 1] = t.y;
-            v[4 * q + 2] = t.z;
-            v[4 * q + 3] = t.w;
-        }
-    } else if constexpr (VEC && sizeof(T) == 8) {
-        static_assert(S % 2 == 0, "double slice must be a multiple of 2");
-        const double2 *p = reinterpret_cast<const double2 *>(row + c0);
-#pragma unroll
-        for (int q = 0; q < S / 2; ++q) {
-            double2 t = __ldg(p + q);
-            v[2 * q + 0] = t.x;
-            v[2 * q + 1] = t.y;
-        }
-    } else {
-#pragma unroll
-        for (int s = 0; s < S; ++s) v[s] = (c0 + s < k) ? __ldg(row + c0 + s) : T(0);
-    }
-}
-
 }  // namespace glrm

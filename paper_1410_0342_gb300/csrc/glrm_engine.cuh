@@ -1094,8 +1094,10 @@ cudaError_t launch_seg(glrm_s *h, const Orient &o, T *F, const T *W, T *alpha, i
     const uintptr_t at = reinterpret_cast<uintptr_t>(F) | reinterpret_cast<uintptr_t>(W);
     const bool vec = h->k == K && at % 16 == 0;
     // few segments: fewer warps per block, so that they spread over the SMs
-    int warps = kWarpsPerBlock;
-    while (warps > 1 && o.nseg < 152LL * warps) warps /= 2;
+    int warps = kWarpsPerBlock, sms = 0;
+    const cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+    if (e != cudaSuccess) return e;
+    while (warps > 1 && o.nseg < (int64_t)sms * warps) warps /= 2;
     const unsigned nb = blocks_for(o.nseg, warps);
     auto go = [&](auto kern) {
         kern<<<nb, warps * 32, 0, h->stream>>>(
@@ -1121,7 +1123,10 @@ cudaError_t dispatch_seg(glrm_s *h, const Orient &o, T *F, const T *W, T *alpha,
 #define GLRM_SEG_CASE(KK) \
     if (k <= KK) return launch_seg<T, KK, XSTEP>(h, o, F, W, alpha, rk, rw);
     GLRM_SEG_CASE(4)
-    if constexpr (std::is_same<T, double>::value) {  // no padding through the FP64 unit at small ranks
+    // ranks 5 and 6 without padding through the FP64 unit (200 x 100, k = 5, 20
+    // sweeps: 983 us padded to 8, 784 us with this and warp_sum_vec); 7 and 9 to
+    // 11 go padded to 8 and 12
+    if constexpr (std::is_same<T, double>::value) {
         GLRM_SEG_CASE(5)
         GLRM_SEG_CASE(6)
     }

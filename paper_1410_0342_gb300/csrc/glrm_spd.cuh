@@ -59,7 +59,8 @@ struct GramTile {
     }
 };
 
-// Sum over the lanes of a K-lane group (K a power of two, groups aligned).
+// Largest value over the lanes of a K-lane group (K a power of two, groups
+// aligned), on every lane of it.
 template <int K, class T>
 __device__ __forceinline__ T group_max(T v)
 {

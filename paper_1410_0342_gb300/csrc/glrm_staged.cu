@@ -9,23 +9,23 @@
 // no registers, so a warp streams its chunk's entries through a ring of kRing
 // blocks of eight, where the register version keeps one gather in flight and
 // waits on its latency.  200,000 x 20,000 completion table, k = 64: 1.35 -> 0.93
-// ms (X-step) and 1.05 -> 0.84 ms (Y-step).  The same ring with FP32 rows
+// ms (X-step) and 1.05 -> 0.81 ms (Y-step).  The same ring with FP32 rows
 // (twice the bytes) was slower than the registers: 6.0 against 5.0 ms for the
 // 2e8-entry Y-step gradient pass, 6.3 against 3.2 ms for the loss pass, which
 // already fills the L1 pipe.
 #include "glrm_engine.cuh"
-#include "glrm_spd.cuh"
+#include "glrm_tiled.cuh"
 
 namespace glrm {
 
 constexpr int kRing = 8;       // blocks of eight entries in flight per warp
 constexpr int kPassWarps = 4;  // warps per CTA of the streaming pass
 
-template <int K, class WT>
+template <int K>
 struct StLane {
-    static constexpr int S = K / 4;                        // coordinates per lane
-    static constexpr int VW = 16 / (int)sizeof(WT);        // values per 16-byte unit
-    static constexpr int H = S / VW;                       // units per lane
+    static constexpr int S = K / 4;    // coordinates per lane
+    static constexpr int VW = 8;       // values per 16-byte unit
+    static constexpr int H = S / VW;   // units per lane
     static_assert(S % VW == 0, "whole units");
     __device__ static __forceinline__ int coord(int s, int gl) { return VW * ((s / VW) * 4 + gl) + s % VW; }
 };
@@ -39,21 +39,22 @@ template <int N>
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 // A row's coordinates of lane gl, FP32 from global memory (0 beyond k).
-template <int K, class WT>
+template <int K>
 __device__ __forceinline__ void st_own(float (&v)[K / 4], const float *__restrict__ row, int gl, int k)
 {
 #pragma unroll
     for (int s = 0; s < K / 4; ++s) {
-        const int c = StLane<K, WT>::coord(s, gl);
+        const int c = StLane<K>::coord(s, gl);
         v[s] = c < k ? __ldg(row + c) : 0.f;
     }
 }
 
 // Request a row's units of lane gl into its place; units beyond k are zeroed.
-template <int K, class WT>
-__device__ __forceinline__ void st_request(unsigned char *place, const WT *__restrict__ W, int64_t j, int gl, int k)
+template <int K>
+__device__ __forceinline__ void st_request(unsigned char *place, const __nv_bfloat16 *__restrict__ W, int64_t j, int gl,
+                                           int k)
 {
-    using LN = StLane<K, WT>;
+    using LN = StLane<K>;
 #pragma unroll
     for (int h = 0; h < LN::H; ++h) {
         const int c = LN::VW * (4 * h + gl);
@@ -62,26 +63,17 @@ __device__ __forceinline__ void st_request(unsigned char *place, const WT *__res
     }
 }
 
-template <int K, class WT>
+template <int K>
 __device__ __forceinline__ void st_read(float (&w)[K / 4], const unsigned char *place)
 {
-    using LN = StLane<K, WT>;
 #pragma unroll
-    for (int h = 0; h < LN::H; ++h) {
-        if constexpr (sizeof(WT) == 4) {
-            const float4 v = *reinterpret_cast<const float4 *>(place + h * 512);
-            w[4 * h] = v.x;
-            w[4 * h + 1] = v.y;
-            w[4 * h + 2] = v.z;
-            w[4 * h + 3] = v.w;
-        } else {
-            const uint4 v = *reinterpret_cast<const uint4 *>(place + h * 512);
-            const uint32_t t[4] = {v.x, v.y, v.z, v.w};
+    for (int h = 0; h < StLane<K>::H; ++h) {
+        const uint4 v = *reinterpret_cast<const uint4 *>(place + h * 512);
+        const uint32_t t[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                w[8 * h + 2 * q] = __uint_as_float(t[q] << 16);
-                w[8 * h + 2 * q + 1] = __uint_as_float(t[q] & 0xffff0000u);
-            }
+        for (int q = 0; q < 4; ++q) {
+            w[8 * h + 2 * q] = __uint_as_float(t[q] << 16);
+            w[8 * h + 2 * q + 1] = __uint_as_float(t[q] & 0xffff0000u);
         }
     }
 }
@@ -112,15 +104,15 @@ __device__ __forceinline__ void st_axpy(float (&g)[S], float d, const float (&w)
 
 // Partial gradient and loss at F of a warp's chunk; `sel` / `want` as in
 // pass_kernel.  uniform: every column has loss[0].
-template <int K, bool XSTEP, class WT>
+template <int K, bool XSTEP>
 __global__ void __launch_bounds__(kPassWarps * 32)
 staged_pass_kernel(int64_t nchunks, const int4 *__restrict__ chunks, const int32_t *__restrict__ order,
                    const int32_t *__restrict__ idx, const float *__restrict__ val, const float *__restrict__ F,
-                   const WT *__restrict__ W, int k, const LossSpecF *__restrict__ loss, bool uniform,
+                   const __nv_bfloat16 *__restrict__ W, int k, const LossSpecF *__restrict__ loss, bool uniform,
                    float *__restrict__ part_grad, double *__restrict__ part_loss, const int32_t *__restrict__ sel,
                    int want)
 {
-    using LN = StLane<K, WT>;
+    using LN = StLane<K>;
     constexpr int S = LN::S, H = LN::H;
     extern __shared__ __align__(16) unsigned char st_raw[];
     __shared__ float ash[kPassWarps][kRing][32];
@@ -133,7 +125,7 @@ staged_pass_kernel(int64_t nchunks, const int4 *__restrict__ chunks, const int32
     if (sel && ((__ldg(sel + ch.x) != 0) != (want != 0))) return;  // another launch takes this segment
     unsigned char *ring = st_raw + (size_t)wid * kRing * H * 512 + lane * 16;
     float f[S], g[S];
-    st_own<K, WT>(f, F + (int64_t)ch.x * k, gl, k);
+    st_own<K>(f, F + (int64_t)ch.x * k, gl, k);
 #pragma unroll
     for (int s = 0; s < S; ++s) g[s] = 0.f;
     LossSpecF sp = loss[XSTEP ? 0 : ch.x];
@@ -155,7 +147,7 @@ staged_pass_kernel(int64_t nchunks, const int4 *__restrict__ chunks, const int32
         const int j = __shfl_sync(0xffffffffu, ji, src);
         const float a = __shfl_sync(0xffffffffu, ai, src);
         const int r = t & (kRing - 1);
-        if (8 * t + grp < len) st_request<K, WT>(ring + r * H * 512, W, j, gl, k);
+        if (8 * t + grp < len) st_request<K>(ring + r * H * 512, W, j, gl, k);
         ash[wid][r][lane] = a;
         if constexpr (XSTEP) jsh[wid][r][lane] = j;
         if ((t & 3) == 3) {
@@ -176,7 +168,7 @@ staged_pass_kernel(int64_t nchunks, const int4 *__restrict__ chunks, const int32
         const int r = t & (kRing - 1);
         const bool in = 8 * t + grp < len;
         float w[S];
-        st_read<K, WT>(w, ring + r * H * 512);
+        st_read<K>(w, ring + r * H * 512);
         const float u = st_dot<S>(f, w);
         if (in) {
             const float a = ash[wid][r][lane];
@@ -217,8 +209,8 @@ static cudaError_t go_pass(glrm_s *h, const Orient &o, const float *F, const __n
                            const int32_t *sel, int want)
 {
     if (o.nchunks == 0) return cudaSuccess;
-    auto kern = staged_pass_kernel<64, XSTEP, __nv_bfloat16>;
-    constexpr size_t smem = (size_t)kPassWarps * kRing * StLane<64, __nv_bfloat16>::H * 512;
+    auto kern = staged_pass_kernel<64, XSTEP>;
+    constexpr size_t smem = (size_t)kPassWarps * kRing * StLane<64>::H * 512;
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     kern<<<blocks_for(o.nchunks, kPassWarps), kPassWarps * 32, smem, h->stream>>>(

@@ -56,10 +56,9 @@ __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence:
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
 // One lane of a converged warp, by elect.sync.  A region that issues MMAs is
-// entered through it and not through a test of the lane number: the compiler
-// then keeps the MMAs' descriptors in uniform registers.  Twelve MMAs beside
-// four busy warps on the scheduler take 733 cycles to issue against 2572
-// (358 against 644 on an idle SM).
+// entered through it and not through a test of the lane number: twelve MMAs
+// beside four busy warps on the scheduler then take 733 cycles to issue against
+// 2572 (358 against 644 on an idle SM).
 __device__ __forceinline__ bool elect_one()
 {
     uint32_t p;
