@@ -23,7 +23,6 @@ template <int K>
 struct Tri {
     static constexpr int N = K * (K + 1) / 2;  // lower-triangle entries
     static constexpr int P = N + K;            // + right-hand side
-    static constexpr int NP = (N + 31) / 32;   // per lane
 };
 
 // Row r and column c (c <= r) of lower-triangle entry p (row-major order).
@@ -41,8 +40,9 @@ __device__ __forceinline__ void tri_rc(int p, int &r, int &c)
 // touched 32 lines with every load); the 32 / K lane groups take the batch's
 // entries in turn, each accumulating its whole K x K tile in registers
 // (GramTile), and are summed at the end.  On the 100,000 x 20,000 completion
-// table (k = 32, 2e7 entries) 4.5 -> 0.94 (rows) and 4.7 -> 1.02 ms (columns); bound by the FP32
-// multiply-adds of the full square (1,024 per entry).
+// table (k = 32, 2e7 entries) 4.5 -> 0.94 (rows) and 4.7 -> 1.02 ms (columns).
+// Bound by the shared-memory reads of the tiles' operands (that pipe is 79 / 67%
+// busy, the FP32 multiply-adds of the full square, 1,024 per entry, 40 / 37%).
 template <class T, int K>
 __global__ void __launch_bounds__(kAlsWarps * 32)
 als_gram_kernel(int64_t nchunks, const int4 *__restrict__ chunks, const int32_t *__restrict__ idx,
