@@ -650,7 +650,7 @@ def run_form(args):
         line.update({
             "metric": METRIC, "unit": UNIT, "value": nnz * args.steps / (ms_graph / 1e3),
             "config": {"workload": f"{wb.count} instances, m~U[50,5000], n~U[20,500], k in {{4,8,16}}, even "
-                                   "quadratic (ALS, FP64 Cholesky), odd Huber (prox-grad), 30% missing, "
+                                   "quadratic (ALS), odd Huber (prox-grad), 30% missing, "
                                    "gamma=0.1, FP32", "nnz": nnz, "generate_s": gen_s},
             "ms_per_sweep": {"graph": ms_graph / args.steps, "stream": ms_stream / args.steps,
                              "per_instance_launches": ms_inst / args.steps},

@@ -123,9 +123,10 @@ int tiled_width(int k)
 
 // Density from which an FP32 observed set is stored densely (NaN marking the
 // missing cells) and swept by the tensor-core form.  Below it the dense sweeps
-// are still the faster ones on large tables (50,021 x 701, k = 18, 25%: 414
-// against 850 us), but the split products' factors are further from the FP64
-// sweep's there than the sparse paths' (5.1e-7 against 5.2e-8 relative).
+// are still the faster ones on large tables (50,021 x 701, k = 18, 25%: 436
+// against 664 us; 30,000 x 500, k = 8, 30%: 326 against 300), but Yt is further
+// from the FP64 sweep's there than with the sparse paths (7.9e-8 against 3.9e-8
+// relative, 1.2e-7 against 3.8e-8; X 4.4e-8 against 4.2e-8, 4.0e-8 against 5.3e-8).
 constexpr double kDenseAutoDensity = 0.4;
 
 // Pick fused / blocked / chunked for one orientation: fused when the whole
